@@ -315,6 +315,7 @@ static int64_t rec_table_tiles(int64_t ny, int64_t ld) { return wtb_tiles(ny, ld
 static size_t rec_off_bytes(int64_t ny, int64_t ld) { return ((size_t)rec_table_tiles(ny, ld) + 1) * sizeof(int); }
 
 static size_t align16(size_t n) { return (n + 15) / 16 * 16; }
+static size_t align128(size_t n) { return (n + 127) / 128 * 128; }
 
 static int64_t flow_tiles(int64_t ny, int64_t ld) {
   const int64_t t = rec_table_tiles(ny, ld);
@@ -323,7 +324,8 @@ static int64_t flow_tiles(int64_t ny, int64_t ld) {
 
 size_t energy_ws_bytes(int64_t ny, int64_t ld) {
   return 256 + align16((size_t)energy_slots(ny, ld) * sizeof(double)) +
-         align16(rec_off_bytes(ny, ld)) + (size_t)kWtbMaxReceivers * sizeof(int4) + flow_bytes(flow_tiles(ny, ld));
+         align16(rec_off_bytes(ny, ld)) + (size_t)kWtbMaxReceivers * sizeof(int4) + align128(flow_bytes(flow_tiles(ny, ld))) +
+         (res_bytes(ny, ld) ? res_bytes(ny, ld) + 128 : 0);
 }
 
 EnergyWs energy_ws_carve(void* ws, size_t bytes, int64_t ny, int64_t ld) {
@@ -341,6 +343,8 @@ EnergyWs energy_ws_carve(void* ws, size_t bytes, int64_t ny, int64_t ld) {
     e.rec_ent_cap = kWtbMaxReceivers;
     e.flow = t + off + (size_t)kWtbMaxReceivers * sizeof(int4);
     e.flow_tiles_cap = flow_tiles(ny, ld);
+    if (res_bytes(ny, ld))
+      e.res = (void*)align128((size_t)e.flow + flow_bytes(e.flow_tiles_cap));
   }
   return e;
 }

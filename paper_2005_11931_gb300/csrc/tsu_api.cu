@@ -304,6 +304,9 @@ int tsu_step_workspace(const tsu_grid* g, int dtype, size_t* bytes) {
 }
 
 
+// calls of fewer steps are not worth reading the fields on chip and writing them back
+static constexpr int64_t kResMinSteps = 8;
+
 int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, tsu_state* st, int64_t nsteps,
                const tsu_step_opts* opts, void* ws, size_t ws_bytes, void* stream) {
   g_err[0] = 0;
@@ -351,8 +354,8 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   const bool tb_possible = blocked_base && !o.traces && !o.ckpt;
   if (o.kernel == 2 && !wtb_possible)
     return fail(TSU_EINVAL, "kernel 2 needs FP32, nbuf = 4, a workspace and checkpoints on its launch boundaries");
-  const bool flow_possible = blocked_base && st->form == TSU_FORM_INCREMENT && !o.traces && !o.ckpt &&
-                             (o.tdepth == 0 || o.tdepth == 4);
+  const bool flow_base = blocked_base && st->form == TSU_FORM_INCREMENT && (o.tdepth == 0 || o.tdepth == 4);
+  const bool flow_possible = flow_base && !o.traces && !o.ckpt;
   if (o.kernel == 4 && !flow_possible)
     return fail(TSU_EINVAL, "kernel 4 needs FP32 in the increment form, nbuf = 4, a workspace, depth 4 and no "
                             "traces or checkpoints");
@@ -373,12 +376,35 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   const size_t field_bytes = (size_t)g->ny * g->ld * elem_size(dtype);
   cudaStream_t s = (cudaStream_t)stream;
   int64_t k = 0;
-  if (use_wtb && o.traces) {
+  if (o.kernel == 0 && o.rows == 0 && flow_base && !o.ckpt && nsteps >= kResMinSteps &&
+      (!o.traces || o.nrec <= tsu::kResMaxRec)) {
+    // grids whose fields fit on chip: every step of the call in one cooperative launch.  With the
+    // energy, the last nsteps % 4 steps go one per pass as after the blocked passes (the one-step
+    // pass rounds the energy's terms differently)
+    const int64_t nres = o.energy ? nsteps / 4 * 4 : nsteps;
+    const int f1 = scratch_index(st, -1), f2 = scratch_index(st, f1);
+    void* const uu[2] = {st->buf[st->cur], st->buf[f1]};
+    void* const vv[2] = {st->buf[st->aux], st->buf[f2]};
+    bool ran = false;
+    int last = 0;
+    cudaError_t e = tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, o.energy, ews, nres, s, o.nrec, o.rec_idx,
+                                         o.traces, &ran, &last);
+    if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n resident launch");
+    if (ran) {
+      if (last == 1) {
+        st->cur = f1;
+        st->aux = f2;
+      }
+      st->step += nres;
+      k = nres;
+    }
+  }
+  if (k == 0 && use_wtb && o.traces) {
     cudaError_t e = tsu::launch_wtb_rec_table(sg, wrows, o.rec_idx, o.nrec, ews, s);
     if (e == cudaSuccess) e = tsu::launch_wtb_trace_edges(sg, o.rec_idx, o.nrec, o.traces, nsteps / wdepth * wdepth, s);
     if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n receiver table");
   }
-  if (use_wtb && flow_possible && (o.kernel == 4 || (o.kernel == 0 && tsu::wtb_flow_preferred(g->ny, g->ld)))) {
+  if (k == 0 && use_wtb && flow_possible && (o.kernel == 4 || (o.kernel == 0 && tsu::wtb_flow_preferred(g->ny, g->ld)))) {
     // kernel 4, and the automatic choice for grids of 2K to 12K per side: every pass of the call
     // in one persistent launch (the same states; 2048^2 611 against 481 GLUPS, 4096^2 988 against
     // 826, 8192^2 1030-1052 against 963)

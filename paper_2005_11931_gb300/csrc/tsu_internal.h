@@ -40,6 +40,7 @@ struct EnergyWs {
   int32_t rec_ent_cap;
   void* flow;              // the persistent warp-blocked pass's counters and energy partials, or nullptr
   int64_t flow_tiles_cap;  // tiles it holds room for
+  void* res;               // the resident pass's rims and energy partials, or nullptr
 };
 
 // The persistent warp-blocked pass (k_leapfrog_wtb_flow): energy partials of kFlowSlots passes
@@ -52,6 +53,19 @@ inline size_t flow_bytes(int64_t tiles) {
   const size_t t4 = (size_t)(tiles + 3) / 4 * 4;
   return 128 + (t4 * sizeof(int) + 15) / 16 * 16 + (size_t)kFlowSlots * 4 * t4 * sizeof(double);
 }
+
+// The resident pass (k_step_res.cu): one CTA per SM, every step of a call in one cooperative launch,
+// for grids whose fields fit on chip.  Its region of the workspace holds the rims that the CTAs
+// exchange and a ring of energy partials.
+constexpr int kResMaxCtas = 160;
+constexpr int32_t kResMaxRec = 512;  // receivers a CTA keeps in its list
+size_t res_bytes(int64_t ny, int64_t ld);  // 0: the grid does not fit
+// nsteps steps (FP32, increment form): from (u, v)[0], using (u, v)[1] as the other pair;
+// the state ends up in (u, v)[*last].  energy and traces per step, or nullptr.  *ran = false and
+// nothing enqueued when the device, the workspace or the grid do not allow it.
+cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
+                            double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
+                            const int64_t* rec_idx, void* traces, bool* ran, int* last);
 
 // receivers the warp-blocked pass records itself (longer lists go one step per pass)
 constexpr int32_t kWtbMaxReceivers = 2048;
