@@ -28,7 +28,7 @@ struct AccOf<float> { using type = float; };
 template <>
 struct AccOf<double> { using type = double; };
 
-// MODE 0 (kAdjStep):     lam_out = (2 lam_c - lam_pp) + B lam_c          (the recursion)
+// (kAdjStep, the recursion itself, is FP64 only: k_step64.cu)
 // MODE 1 (kAdjStart):    lam_out = (lam_c - lam_pp) + B lam_c / 2 = dJ/du0; g_u1 = tau lam_c
 // MODE 2 (kAdjStepInc):  lam_pp holds mu^{n+1}: mu_out = mu^{n+1} + B lam_c (may be lam_pp itself:
 //                        every node reads only its own mu), lam_out = lam_c + mu_out
@@ -98,9 +98,7 @@ __global__ void __launch_bounds__(128) k_adjoint_pass(const int32_t nx, const in
       const T b = ar.b(hxv.a[e], hxl, hyv.a[e], hym.a[e], lc.a[e], xl, xr, ln.a[e], lm.a[e]);
       const bool interior = (i >= 1) && (i <= nx - 2);
       T val;
-      if constexpr (MODE == 0) {
-        val = ar.lf(lc.a[e], lp.a[e], b);
-      } else if constexpr (MODE == 2) {
+      if constexpr (MODE == 2) {
         const T mu = ar.add(lp.a[e], b);
         mo.a[e] = interior ? mu : T(0);
         val = ar.add(lc.a[e], mu);
@@ -162,14 +160,21 @@ __global__ void __launch_bounds__(128) k_adjoint_pass(const int32_t nx, const in
   }
 }
 
-// Receivers grouped by the CTA of the adjoint pass that owns their node (interior nodes only),
-// in receiver order: off[ncta + 1], ord[nrec].  One thread; nrec and ncta are small.
-__global__ void k_rec_bucket(const int32_t nx, const int32_t ny, const int64_t ld, const int64_t* idx,
-                             const int32_t nrec, const int64_t cols_per_cta, const int rows, const int64_t gridx,
-                             const int64_t ncta, int* off, int* ord, int* cta_of) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int64_t c = 0; c <= ncta; ++c) off[c] = 0;
-  for (int r = 0; r < nrec; ++r) {
+// Receivers grouped by the CTA (or tile) of the adjoint pass that owns their node (interior nodes
+// only), in receiver order: off[ncta + 1], ord[nrec].  One CTA: counts, a scan, and each receiver
+// placed by its rank among the earlier ones of its bucket (one thread alone took 0.1 ms at 1700
+// tiles).
+__global__ void __launch_bounds__(1024) k_rec_bucket(const int32_t nx, const int32_t ny, const int64_t ld,
+                                                     const int64_t* idx, const int32_t nrec,
+                                                     const int64_t cols_per_cta, const int rows, const int64_t gridx,
+                                                     const int64_t ncta, int* off, int* ord, int* cta_of) {
+  __shared__ int wsum[32];
+  __shared__ int carry;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t c = threadIdx.x; c <= ncta; c += blockDim.x) off[c] = 0;
+  if (threadIdx.x == 0) carry = 0;
+  __syncthreads();
+  for (int r = threadIdx.x; r < nrec; r += blockDim.x) {
     const int64_t q = idx[r];
     int c = -1;
     if (q >= 0 && q < (int64_t)ny * ld) {
@@ -177,14 +182,41 @@ __global__ void k_rec_bucket(const int32_t nx, const int32_t ny, const int64_t l
       if (i >= 1 && i <= nx - 2 && j >= 1 && j <= ny - 2) c = (int)(((j - 1) / rows) * gridx + i / cols_per_cta);
     }
     cta_of[r] = c;
-    if (c >= 0) off[c + 1] += 1;
+    if (c >= 0) atomicAdd(&off[c + 1], 1);
   }
-  for (int64_t c = 0; c < ncta; ++c) off[c + 1] += off[c];
-  // stable fill with off[c] as the cursor of bucket c, then shift the cursors back to the starts
-  for (int r = 0; r < nrec; ++r)
-    if (cta_of[r] >= 0) ord[off[cta_of[r]]++] = r;
-  for (int64_t c = ncta; c >= 1; --c) off[c] = off[c - 1];
-  off[0] = 0;
+  __syncthreads();
+  for (int64_t base = 1; base <= ncta; base += blockDim.x) {  // inclusive scan of off[1 .. ncta]
+    const int64_t c = base + threadIdx.x;
+    int v = c <= ncta ? off[c] : 0;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += n;
+    }
+    if (lane == 31) wsum[w] = v;
+    __syncthreads();
+    if (w == 0) {
+      int x = wsum[lane];
+      for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += n;
+      }
+      wsum[lane] = x;
+    }
+    __syncthreads();
+    const int incl = v + (w > 0 ? wsum[w - 1] : 0) + carry;
+    if (c <= ncta) off[c] = incl;
+    __syncthreads();
+    if (threadIdx.x == blockDim.x - 1) carry = incl;
+    __syncthreads();
+  }
+  for (int r = threadIdx.x; r < nrec; r += blockDim.x) {
+    const int c = cta_of[r];
+    if (c < 0) continue;
+    int rank = 0;
+    if (off[c + 1] - off[c] > 1)
+      for (int t = 0; t < r; ++t) rank += cta_of[t] == c;
+    ord[off[c] + rank] = r;
+  }
 }
 
 // lam[rec_idx[r]] += g[r] for interior receiver nodes (boundary receivers record a constant 0)
@@ -218,14 +250,28 @@ typename AdjArithOf<T>::type arith(const StencilGeom& g) {
 
 }  // namespace
 
-void adjoint_pass_shape(const StencilGeom& g, int dtype, int64_t* gridx, int64_t* gridy, int* rows,
-                        int64_t* cols_per_cta) {
+namespace {
+void pass_shape(const StencilGeom& g, int dtype, int64_t* gridx, int64_t* gridy, int* rows, int64_t* cols_per_cta) {
   const int64_t cpc = (int64_t)128 * (dtype == TSU_F32 ? 4 : 2);
   const int r = auto_rows(g.ld, g.ny, cpc);
   *cols_per_cta = cpc;
   *rows = r;
   *gridx = (g.ld + cpc - 1) / cpc;
   *gridy = (g.ny - 2 + r - 1) / r;
+}
+}  // namespace
+
+// the units the receivers are bucketed by: CTAs of k_adjoint_pass (FP32), tiles of k_adjoint64
+void adjoint_pass_shape(const StencilGeom& g, int dtype, int64_t* gridx, int64_t* gridy, int* rows,
+                        int64_t* cols_per_cta) {
+  if (dtype == TSU_F32) {
+    pass_shape(g, dtype, gridx, gridy, rows, cols_per_cta);
+    return;
+  }
+  *rows = step64_rows(g.nx, g.ny);
+  *cols_per_cta = kStep64Cols;
+  *gridx = step64_strips(g.nx);
+  *gridy = (g.ny - 2 + *rows - 1) / *rows;
 }
 
 namespace {
@@ -245,20 +291,20 @@ cudaError_t pass_t(const StencilGeom& g, int mode, const void* hx, const void* h
                    const RecBuckets& rb, cudaStream_t s) {
   int64_t gx_, gy_, cpc;
   int rows;
-  adjoint_pass_shape(g, sizeof(T) == 4 ? TSU_F32 : TSU_F64, &gx_, &gy_, &rows, &cpc);
+  pass_shape(g, sizeof(T) == 4 ? TSU_F32 : TSU_F64, &gx_, &gy_, &rows, &cpc);
   dim3 grid((unsigned)gx_, (unsigned)gy_);
   const bool start = mode == kAdjStart || mode == kAdjStartInc;
   const T w = start ? T(0.5) : T(1);
   const T gwx = -(T)g.cx * w, gwy = -(T)g.cy * w;
   switch (mode) {
-    case kAdjStep:
-      pass_mode<T, 0>(grid, g, gwx, gwy, hx, hy, lam, lam_pp, lam_out, mu_out, u, gx, gy, g_u1, rows, rb, s);
-      break;
     case kAdjStart:
       pass_mode<T, 1>(grid, g, gwx, gwy, hx, hy, lam, lam_pp, lam_out, mu_out, u, gx, gy, g_u1, rows, rb, s);
       break;
     case kAdjStepInc:
-      pass_mode<T, 2>(grid, g, gwx, gwy, hx, hy, lam, lam_pp, lam_out, mu_out, u, gx, gy, g_u1, rows, rb, s);
+      if constexpr (sizeof(T) == 4)
+        pass_mode<T, 2>(grid, g, gwx, gwy, hx, hy, lam, lam_pp, lam_out, mu_out, u, gx, gy, g_u1, rows, rb, s);
+      else
+        return cudaErrorInvalidValue;
       break;
     case kAdjStartInc:
       pass_mode<T, 3>(grid, g, gwx, gwy, hx, hy, lam, lam_pp, lam_out, mu_out, u, gx, gy, g_u1, rows, rb, s);
@@ -275,13 +321,15 @@ cudaError_t launch_rec_bucket(const StencilGeom& g, int dtype, const int64_t* id
   int64_t gx_, gy_, cpc;
   int rows;
   adjoint_pass_shape(g, dtype, &gx_, &gy_, &rows, &cpc);
-  k_rec_bucket<<<1, 32, 0, s>>>(g.nx, g.ny, g.ld, idx, nrec, cpc, rows, gx_, gx_ * gy_, off, ord, cta_of);
+  k_rec_bucket<<<1, 1024, 0, s>>>(g.nx, g.ny, g.ld, idx, nrec, cpc, rows, gx_, gx_ * gy_, off, ord, cta_of);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint_pass(const StencilGeom& g, int dtype, int mode, const void* hx, const void* hy,
                                 const void* lam, const void* lam_pp, void* lam_out, void* mu_out, const void* u,
                                 void* gx, void* gy, void* g_u1, const RecBuckets& rb, cudaStream_t s) {
+  if (mode == kAdjStep)
+    return dtype == TSU_F64 ? launch_adjoint64(g, hx, hy, lam, (void*)lam_pp, u, gx, gy, rb, s) : cudaErrorInvalidValue;
   return dtype == TSU_F32 ? pass_t<float>(g, mode, hx, hy, lam, lam_pp, lam_out, mu_out, u, gx, gy, g_u1, rb, s)
                           : pass_t<double>(g, mode, hx, hy, lam, lam_pp, lam_out, mu_out, u, gx, gy, g_u1, rb, s);
 }

@@ -11,8 +11,7 @@
 // The same pass optionally yields the discrete energy of the pair it reads (the leapfrog analogue
 // of (CL-01), Theorem 2.1), receiver samples and a checkpoint copy.
 //
-// FP64 fields are evaluated with explicitly rounded operations in the order of the definition
-// (no fused multiply-add), FP32 fields with fused multiply-adds.
+// This file runs FP32 fields, with fused multiply-adds; the FP64 steps are k_step64.cu's.
 #include "stencil_common.cuh"
 
 namespace tsu {
@@ -271,8 +270,7 @@ cudaError_t launch_step(const StencilGeom& g, int dtype, int form, const void* h
   if (dtype == TSU_F32)
     return form == TSU_FORM_STANDARD ? step_t<float, 0>(g, hx, hy, u_prev, u_cur, v, u_next, o, store, rows, s)
                                      : step_t<float, 1>(g, hx, hy, u_prev, u_cur, v, u_next, o, store, rows, s);
-  return form == TSU_FORM_STANDARD ? step_t<double, 0>(g, hx, hy, u_prev, u_cur, v, u_next, o, store, rows, s)
-                                   : step_t<double, 1>(g, hx, hy, u_prev, u_cur, v, u_next, o, store, rows, s);
+  return launch_step64(g, form, hx, hy, u_prev, u_cur, v, u_next, o, store, rows, s);
 }
 
 cudaError_t launch_init(const StencilGeom& g, int dtype, int form, const void* hx, const void* hy, const void* u0,
@@ -306,7 +304,9 @@ cudaError_t launch_init(const StencilGeom& g, int dtype, int form, const void* h
 static int64_t energy_slots(int64_t ny, int64_t ld) {
   const int64_t plain = ((ld + 127) / 128) * (ny > 2 ? ny - 2 : 1);
   const int64_t tb = tb_energy_slots(ny, ld, 8, 16);
-  return plain > tb ? plain : tb;
+  const int64_t f64 = ((ld + 30) / 31 * (ny > 2 ? ny - 2 : 1) + 3) / 4;  // k_step64.cu, a row per tile
+  const int64_t most = plain > tb ? plain : tb;
+  return most > f64 ? most : f64;
 }
 
 // the warp-blocked pass's receiver table: tiles + 1 offsets (at least 16 rows per chunk) and
@@ -343,8 +343,10 @@ EnergyWs energy_ws_carve(void* ws, size_t bytes, int64_t ny, int64_t ld) {
     e.rec_ent_cap = kWtbMaxReceivers;
     e.flow = t + off + (size_t)kWtbMaxReceivers * sizeof(int4);
     e.flow_tiles_cap = flow_tiles(ny, ld);
-    if (res_bytes(ny, ld))
+    if (res_bytes(ny, ld)) {
       e.res = (void*)align128((size_t)e.flow + flow_bytes(e.flow_tiles_cap));
+      e.res_size = res_bytes(ny, ld);
+    }
   }
   return e;
 }

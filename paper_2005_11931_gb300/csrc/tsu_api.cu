@@ -460,10 +460,19 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
       st->step += tdepth;
     }
   }
+  // FP64 steps with the energy: the CTAs' partials of several steps are kept (in the region the FP32
+  // resident pass has) and summed by one launch, instead of by the last CTA of every step, which on
+  // small grids costs as much as the step
+  const int64_t ctas64 = dtype == TSU_F64 ? tsu::step64_ctas(g->nx, g->ny, o.rows) : 0;
+  const int64_t keep = ctas64 > 0 && ctas64 <= 1024 && o.energy && ews.res
+                           ? std::min<int64_t>(256, (int64_t)(ews.res_size / (ctas64 * sizeof(double))))
+                           : 0;
+  int64_t kept = 0;
   for (; k < nsteps; ++k) {
     tsu::PassOut po{};
     po.energy = o.energy ? o.energy + k : nullptr;
     po.ews = ews;
+    if (keep > 1) po.defer = (double*)ews.res + kept * ctas64;
     po.nrec = o.nrec;
     po.rec_idx = o.rec_idx;
     po.trace = o.traces ? (char*)o.traces + (size_t)k * o.nrec * elem_size(dtype) : nullptr;
@@ -481,6 +490,10 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
       const int f = scratch_index(st, -1);
       e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, nullptr, st->buf[st->cur], st->buf[st->aux],
                            st->buf[f], po, true, (use_tb || use_wtb) ? 0 : o.rows, s);
+    }
+    if (e == cudaSuccess && po.defer && (++kept == keep || k + 1 == nsteps)) {
+      e = tsu::launch_energy64(sg, (const double*)ews.res, ctas64, kept, o.energy + (k + 1 - kept), s);
+      kept = 0;
     }
     if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n launch");
     if (st->form == TSU_FORM_STANDARD) {

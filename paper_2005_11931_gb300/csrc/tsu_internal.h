@@ -41,6 +41,7 @@ struct EnergyWs {
   void* flow;              // the persistent warp-blocked pass's counters and energy partials, or nullptr
   int64_t flow_tiles_cap;  // tiles it holds room for
   void* res;               // the resident pass's rims and energy partials, or nullptr
+  size_t res_size;
 };
 
 // The persistent warp-blocked pass (k_leapfrog_wtb_flow): energy partials of kFlowSlots passes
@@ -120,13 +121,14 @@ struct PassOut {
   void* trace;              // nrec elements, or nullptr
   void* ckpt_a;             // checkpoint slot field 0 (u^{n-1} or u^n), or nullptr
   void* ckpt_b;             // checkpoint slot field 1
+  double* defer;            // FP64: per-CTA energy partials go here, summed later (launch_energy64)
 };
 
 cudaError_t launch_init(const StencilGeom& g, int dtype, int form, const void* hx, const void* hy,
                         const void* u0, const void* u1, tsu_state* st, cudaStream_t s);
 
-// CTAs of one launch of the one-step pass (launch_step) for this grid, element type and rows per
-// CTA (rows <= 0: the automatic choice): one energy partial sum each.
+// CTAs of one launch of the register-streaming pass for this grid, element type and rows per CTA
+// (rows <= 0: the automatic choice).
 int64_t one_step_ctas(int64_t ld, int64_t ny, int dtype, int rows);
 
 // One leapfrog pass (standard or increment form) over the interior; store=false computes only
@@ -134,6 +136,31 @@ int64_t one_step_ctas(int64_t ld, int64_t ny, int dtype, int rows);
 cudaError_t launch_step(const StencilGeom& g, int dtype, int form, const void* hx, const void* hy,
                         const void* u_prev, const void* u_cur, void* v, void* u_next, const PassOut& o,
                         bool store, int rows, cudaStream_t s);
+
+// Receivers bucketed by the adjoint-pass CTA (FP64: tile) owning their node (off[ncta+1], ord[nrec]) and the
+// values g[r] injected into lam^n by that CTA after its stores; off == nullptr: no injection.
+struct RecBuckets {
+  const int* off;
+  const int* ord;
+  const int64_t* idx;
+  const void* g;
+};
+
+// FP64 steps (k_step64.cu), one per launch: tiles of 31 columns x rows (rows <= 0: step64_rows), one warp
+// each.  launch_step and launch_adjoint_pass send FP64 fields here.
+constexpr int kStep64Cols = 31;
+int step64_strips(int64_t nx);
+int step64_rows(int64_t nx, int64_t ny);
+int64_t step64_ctas(int64_t nx, int64_t ny, int rows);  // one energy partial each
+cudaError_t launch_step64(const StencilGeom& g, int form, const void* hx, const void* hy, const void* u_prev,
+                          const void* u_cur, void* v, void* u_next, const PassOut& o, bool store, int rows,
+                          cudaStream_t s);
+// energy[n] of nsteps steps from their partials part[n][ncta] (PassOut.defer)
+cudaError_t launch_energy64(const StencilGeom& g, const double* part, int64_t ncta, int64_t nsteps, double* energy,
+                            cudaStream_t s);
+// one reverse step: lam^n over lam_pp = lam^{n+2}; receivers bucketed by tile
+cudaError_t launch_adjoint64(const StencilGeom& g, const void* hx, const void* hy, const void* lam, void* lam_pp,
+                             const void* u, void* gx, void* gy, const RecBuckets& rb, cudaStream_t s);
 
 // Temporally blocked FP32 pass (k_step_tb.cu): k in {4, 8} steps per launch.
 bool tb_supported_depth(int k);
@@ -195,14 +222,6 @@ cudaError_t launch_step_tb_batched(int form, int k, const void* probs_dev, const
                                    cudaStream_t s);
 
 // Adjoint (k_adjoint.cu).
-// Receivers bucketed by the adjoint-pass CTA owning their node (off[ncta+1], ord[nrec]) and the
-// values g[r] injected into lam^n by that CTA after its stores; off == nullptr: no injection.
-struct RecBuckets {
-  const int* off;
-  const int* ord;
-  const int64_t* idx;
-  const void* g;
-};
 void adjoint_pass_shape(const StencilGeom& g, int dtype, int64_t* gridx, int64_t* gridy, int* rows,
                         int64_t* cols_per_cta);
 cudaError_t launch_rec_bucket(const StencilGeom& g, int dtype, const int64_t* idx, int32_t nrec, int* off, int* ord,

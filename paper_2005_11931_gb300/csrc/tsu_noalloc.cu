@@ -110,6 +110,9 @@ int tsu_step_n_noalloc(const tsu_grid* g, int dtype, double tau, const tsu_mediu
   sg.cy = tau * tau / (g->dy * g->dy);
   sg.tau = tau;
   sg.dxdy = g->dx * g->dy;
+  // FP64 tiles are narrower than the count above assumes: more rows each where that is too many
+  int rows = kNoallocRows;
+  while (dtype == TSU_F64 && tsu::step64_ctas(g->nx, g->ny, rows) > kNoallocPartials) rows *= 2;
   for (int64_t k = 0; k < nsteps; ++k) {
     tsu::PassOut po{};
     po.energy = energy ? energy + k : nullptr;
@@ -117,13 +120,13 @@ int tsu_step_n_noalloc(const tsu_grid* g, int dtype, double tau, const tsu_mediu
     cudaError_t e;
     if (st->form == TSU_FORM_STANDARD) {
       e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, st->buf[st->aux], st->buf[st->cur], nullptr,
-                           st->buf[st->aux], po, true, kNoallocRows, s);
+                           st->buf[st->aux], po, true, rows, s);
     } else {
       int f = -1;
       for (int b = 0; b < st->nbuf && f < 0; ++b)
         if (b != st->cur && b != st->aux) f = b;
       e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, nullptr, st->buf[st->cur], st->buf[st->aux],
-                           st->buf[f], po, true, kNoallocRows, s);
+                           st->buf[f], po, true, rows, s);
       if (e == cudaSuccess) st->cur = f;
     }
     if (e != cudaSuccess) return na_fail(TSU_ECUDA, cudaGetErrorString(e));
