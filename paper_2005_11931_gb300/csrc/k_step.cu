@@ -317,6 +317,12 @@ static size_t rec_off_bytes(int64_t ny, int64_t ld) { return ((size_t)rec_table_
 static size_t align16(size_t n) { return (n + 15) / 16 * 16; }
 static size_t align128(size_t n) { return (n + 127) / 128 * 128; }
 
+// the resident passes' region (FP32 or FP64)
+static size_t res_region(int64_t ny, int64_t ld) {
+  const size_t a = res_bytes(ny, ld), b = res64_bytes(ny, ld);
+  return a > b ? a : b;
+}
+
 static int64_t flow_tiles(int64_t ny, int64_t ld) {
   const int64_t t = rec_table_tiles(ny, ld);
   return t < kFlowMaxTiles ? t : kFlowMaxTiles;
@@ -325,7 +331,7 @@ static int64_t flow_tiles(int64_t ny, int64_t ld) {
 size_t energy_ws_bytes(int64_t ny, int64_t ld) {
   return 256 + align16((size_t)energy_slots(ny, ld) * sizeof(double)) +
          align16(rec_off_bytes(ny, ld)) + (size_t)kWtbMaxReceivers * sizeof(int4) + align128(flow_bytes(flow_tiles(ny, ld))) +
-         (res_bytes(ny, ld) ? res_bytes(ny, ld) + 128 : 0);
+         (res_region(ny, ld) ? res_region(ny, ld) + 128 : 0);
 }
 
 EnergyWs energy_ws_carve(void* ws, size_t bytes, int64_t ny, int64_t ld) {
@@ -343,9 +349,9 @@ EnergyWs energy_ws_carve(void* ws, size_t bytes, int64_t ny, int64_t ld) {
     e.rec_ent_cap = kWtbMaxReceivers;
     e.flow = t + off + (size_t)kWtbMaxReceivers * sizeof(int4);
     e.flow_tiles_cap = flow_tiles(ny, ld);
-    if (res_bytes(ny, ld)) {
+    if (res_region(ny, ld)) {
       e.res = (void*)align128((size_t)e.flow + flow_bytes(e.flow_tiles_cap));
-      e.res_size = res_bytes(ny, ld);
+      e.res_size = res_region(ny, ld);
     }
   }
   return e;

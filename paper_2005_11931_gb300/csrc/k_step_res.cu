@@ -711,7 +711,7 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
     if ((flow ? wtb_flow_rows(g.ny, g.ld) : wtb_auto_rows(g.ny, g.ld, kResK)) != kResChain) return cudaSuccess;
   }
   const int rows = res_rows(g.ny, g.ld, energy != nullptr, &k);
-  if (rows == 0 || !ews.res || !ews.status || nsteps < 1 || nsteps >= (int64_t)1 << 31 ||
+  if (rows == 0 || !ews.res || ews.res_size < res_bytes(g.ny, g.ld) || !ews.status || nsteps < 1 || nsteps >= (int64_t)1 << 31 ||
       (traces && nrec > kResMaxRec))
     return cudaSuccess;
   ResArgs a{};

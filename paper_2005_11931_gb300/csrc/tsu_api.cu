@@ -399,6 +399,17 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
       k = nres;
     }
   }
+  if (o.kernel == 0 && o.rows == 0 && dtype == TSU_F64 && st->form == TSU_FORM_STANDARD && have_ws && !o.ckpt &&
+      nsteps >= kResMinSteps && (!o.traces || o.nrec <= tsu::kResMaxRec)) {
+    bool ran = false;
+    cudaError_t e = tsu::launch_step_res64(sg, m->hx, m->hy, st->buf[st->cur], st->buf[st->aux], o.energy, ews, nsteps,
+                                           s, o.nrec, o.rec_idx, o.traces, &ran);
+    if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n resident FP64 launch");
+    if (ran) {
+      st->step += nsteps;
+      return TSU_OK;
+    }
+  }
   if (k == 0 && use_wtb && o.traces) {
     cudaError_t e = tsu::launch_wtb_rec_table(sg, wrows, o.rec_idx, o.nrec, ews, s);
     if (e == cudaSuccess) e = tsu::launch_wtb_trace_edges(sg, o.rec_idx, o.nrec, o.traces, nsteps / wdepth * wdepth, s);

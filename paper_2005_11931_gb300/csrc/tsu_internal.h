@@ -68,6 +68,13 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
                             double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
                             const int64_t* rec_idx, void* traces, bool* ran, int* last);
 
+// The same for FP64 grids of up to about 750^2 in the standard form (k_step_res64.cu): u = u^n and
+// p = u^{n-1} are updated in place.
+size_t res64_bytes(int64_t ny, int64_t ld);
+cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* hy, void* u, void* p, double* energy,
+                              const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
+                              const int64_t* rec_idx, void* traces, bool* ran);
+
 // receivers the warp-blocked pass records itself (longer lists go one step per pass)
 constexpr int32_t kWtbMaxReceivers = 2048;
 
