@@ -16,7 +16,7 @@
 // nodes and step, 46 of them FP32 arithmetic; streaming tiles through shared memory and register
 // windows, as k_step_wtb.cu does, takes 100 to 176), and one exchange, about 2 us, per four steps.
 // Measured (GB300, us per step, before and after): 769^2 with receivers 4.1 and 1.35; 1024^2 3.6 and
-// 1.51, 1400^2 4.6 and 2.0, 2048^2 5.9 and 4.7; with the energy 1003 x 517 4.8 and 1.7, 1024^2 4.9 and
+// 1.43, 1400^2 4.6 and 1.9, 2048^2 5.9 and 4.7; with the energy 1003 x 517 4.8 and 1.7, 1024^2 4.9 and
 // 2.0, 1536^2 5.7 and 3.0.
 //
 // All warps run the row code in step (a barrier per step): when only neighbouring warps waited for
@@ -29,6 +29,8 @@
 //   wide:   u in registers, v in shared memory, hx and hy in tensor memory (16 rows x 8 columns
 //           of a warp's quarter of the 32 lanes; a 17th row in shared memory).  Tensor memory is
 //           used as a plain scratchpad (tcgen05.st once, tcgen05.ld per row and step).
+// Wide from 5 rows per warp on: 1200^2 2.50 against 3.12 us per step with the energy, 1400^2 1.90 against
+// 2.01 and 1536^2 2.28 against 3.17 without (the narrow tile spills); no difference at 2 to 4 rows.
 //
 // The arithmetic of a node is that of k_step_wtb.cu operation by operation, so the states equal the
 // other passes' bit for bit, and the energy's terms are added up along the same chains of rows.
@@ -623,11 +625,11 @@ constexpr ResVariant res_variant() {
 // without the energy, then with it
 const ResVariant kResVariants[] = {
     res_variant<2, 2, false, false>(),  res_variant<3, 3, false, false>(), res_variant<4, 2, false, false>(),
-    res_variant<5, 2, false, false>(),  res_variant<6, 2, false, false>(), res_variant<7, 2, false, false>(),
-    res_variant<8, 2, false, false>(),  res_variant<10, 2, false, false>(), res_variant<12, 2, true, false>(),
+    res_variant<5, 2, true, false>(),  res_variant<6, 2, true, false>(), res_variant<7, 2, true, false>(),
+    res_variant<8, 2, true, false>(),  res_variant<10, 2, true, false>(), res_variant<12, 2, true, false>(),
     res_variant<14, 2, true, false>(),  res_variant<17, 2, true, false>(), res_variant<2, 2, false, true>(),
-    res_variant<3, 3, false, true>(),   res_variant<4, 2, false, true>(),  res_variant<5, 2, false, true>(),
-    res_variant<6, 2, false, true>(),   res_variant<8, 2, false, true>(),  res_variant<10, 2, true, true>(),
+    res_variant<3, 3, false, true>(),   res_variant<4, 2, false, true>(),  res_variant<5, 2, true, true>(),
+    res_variant<6, 2, true, true>(),   res_variant<8, 2, true, true>(),  res_variant<10, 2, true, true>(),
     res_variant<12, 2, true, true>()};
 constexpr int kResPlain = 11;  // variants without the energy
 constexpr int kResNumVariants = (int)(sizeof kResVariants / sizeof kResVariants[0]);
