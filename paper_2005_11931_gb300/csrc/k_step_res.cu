@@ -702,9 +702,14 @@ static int res_rows(int64_t ny, int64_t ld, bool energy, int* variant) {
   return 0;
 }
 
+bool res_fits(const StencilGeom& g, bool energy) {
+  int k = 0;
+  return res_rows(g.ny, g.ld, energy, &k) > 0;
+}
+
 cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
                             double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
-                            const int64_t* rec_idx, void* traces, bool* ran, int* last) {
+                            const int64_t* rec_idx, void* traces, bool table, bool* ran, int* last) {
   *ran = false;
   *last = 0;
   int k = 0;
@@ -735,7 +740,7 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
   a.status = ews.status;
   cudaError_t e = cudaSuccess;
   if (traces && nrec > 0) {
-    e = launch_wtb_rec_table(g, rows, rec_idx, nrec, ews, s);
+    if (table) e = launch_wtb_rec_table(g, rows, rec_idx, nrec, ews, s);
     if (e == cudaSuccess) e = launch_wtb_trace_edges(g, rec_idx, nrec, traces, nsteps, s);
     if (e != cudaSuccess) return e;
     a.nrec = nrec;

@@ -310,20 +310,31 @@ size_t res64_bytes(int64_t ny, int64_t ld) {
   return least <= kResMaxCtas ? kR64RimBytes + (size_t)kR64EnergySteps * kResMaxCtas * sizeof(double) : 0;
 }
 
+// The variant and the rows per CTA (one CTA per SM, as many as fit); -1: the grid does not fit.
+static int r64_plan(const StencilGeom& g, const EnergyWs& ews, int64_t* rows) {
+  const int64_t sms = r64_sms(), strips = r64_strips(g.nx), inner = g.ny - 2;
+  if (sms <= 0 || strips < 1 || strips > sms || !ews.res || !ews.status || g.ny >= 1 << 22 ||
+      ews.res_size < kR64RimBytes + (size_t)kR64EnergySteps * kResMaxCtas * sizeof(double))
+    return -1;
+  *rows = (inner + sms / strips - 1) / (sms / strips);
+  const int64_t per_warp = (*rows + kR64Warps - 1) / kR64Warps;
+  for (int k = 0; k < kR64Num; ++k)
+    if (kR64Variants[k].rows >= per_warp) return k;
+  return -1;
+}
+bool res64_fits(const StencilGeom& g, const EnergyWs& ews) {
+  int64_t rows = 0;
+  return r64_plan(g, ews, &rows) >= 0;
+}
+
 cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* hy, void* u, void* p, double* energy,
                               const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
                               const int64_t* rec_idx, void* traces, bool* ran) {
   *ran = false;
-  const int64_t sms = r64_sms(), strips = r64_strips(g.nx), inner = g.ny - 2;
-  if (sms <= 0 || strips < 1 || strips > sms || !ews.res || !ews.status || g.ny >= 1 << 22 ||
-      ews.res_size < kR64RimBytes + (size_t)kR64EnergySteps * kResMaxCtas * sizeof(double) || nsteps >= 1ll << 31 ||
-      (traces && nrec > kResMaxRec))
-    return cudaSuccess;
-  const int64_t rows = (inner + sms / strips - 1) / (sms / strips);  // one CTA per SM, as many as fit
-  const int64_t per_warp = (rows + kR64Warps - 1) / kR64Warps;
-  int k = 0;
-  while (k < kR64Num && kR64Variants[k].rows < per_warp) ++k;
-  if (k == kR64Num) return cudaSuccess;
+  int64_t rows = 0;
+  const int k = r64_plan(g, ews, &rows);
+  if (k < 0 || nsteps >= 1ll << 31 || (traces && nrec > kResMaxRec)) return cudaSuccess;
+  const int64_t strips = r64_strips(g.nx), inner = g.ny - 2;
   R64Args a{};
   a.nx = g.nx;
   a.ny = g.ny;

@@ -304,6 +304,18 @@ int tsu_step_workspace(const tsu_grid* g, int dtype, size_t* bytes) {
 }
 
 
+// the state at step n = 1 + c every into slot c: (u^{n-1}, u^n) or, in the increment form, (u^n, v^n)
+static cudaError_t checkpoint(const tsu_state* st, const tsu_step_opts& o, size_t field_bytes, cudaStream_t s) {
+  const int64_t c = (st->step - 1) / o.ckpt_every;
+  if (c >= o.ckpt_slots) return cudaSuccess;
+  char* slot = (char*)o.ckpt + (size_t)c * 2 * field_bytes;
+  const bool standard = st->form == TSU_FORM_STANDARD;
+  cudaError_t e = cudaMemcpyAsync(slot, st->buf[standard ? st->aux : st->cur], field_bytes, cudaMemcpyDeviceToDevice, s);
+  if (e != cudaSuccess) return e;
+  return cudaMemcpyAsync(slot + field_bytes, st->buf[standard ? st->cur : st->aux], field_bytes,
+                         cudaMemcpyDeviceToDevice, s);
+}
+
 // calls of fewer steps are not worth reading the fields on chip and writing them back
 static constexpr int64_t kResMinSteps = 8;
 
@@ -376,43 +388,46 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   const size_t field_bytes = (size_t)g->ny * g->ld * elem_size(dtype);
   cudaStream_t s = (cudaStream_t)stream;
   int64_t k = 0;
-  if (o.kernel == 0 && o.rows == 0 && flow_base && !o.ckpt && nsteps >= kResMinSteps &&
-      (!o.traces || o.nrec <= tsu::kResMaxRec)) {
-    // grids whose fields fit on chip: every step of the call in one cooperative launch.  With the
-    // energy, the last nsteps % 4 steps go one per pass as after the blocked passes (the one-step
-    // pass rounds the energy's terms differently)
-    const int64_t nres = o.energy ? nsteps / 4 * 4 : nsteps;
-    const int f1 = scratch_index(st, -1), f2 = scratch_index(st, f1);
-    void* const uu[2] = {st->buf[st->cur], st->buf[f1]};
-    void* const vv[2] = {st->buf[st->aux], st->buf[f2]};
-    bool ran = false;
-    int last = 0;
-    cudaError_t e = tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, o.energy, ews, nres, s, o.nrec, o.rec_idx,
-                                         o.traces, &ran, &last);
-    if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n resident launch");
-    if (ran) {
+  // Grids whose fields fit on chip: every step up to the next checkpoint in one cooperative launch.  FP32
+  // with the energy: the last nsteps % 4 steps go one per pass as after the blocked passes (the one-step
+  // pass rounds the energy's terms differently), and with checkpoints too the blocked passes run.
+  const bool res32 = flow_base && !(o.energy && o.ckpt);
+  const bool res64 = dtype == TSU_F64 && st->form == TSU_FORM_STANDARD && have_ws;
+  if (o.kernel == 0 && o.rows == 0 && (res32 || res64) && (!o.traces || o.nrec <= tsu::kResMaxRec)) {
+    const int64_t nres = res32 && o.energy ? nsteps / 4 * 4 : nsteps;
+    bool ran = true;
+    while (ran && k < nres) {
+      const int64_t due = o.ckpt ? ((st->step - 1) % o.ckpt_every + o.ckpt_every) % o.ckpt_every : 0;  // 0: now
+      const int64_t n = o.ckpt && o.ckpt_every - due < nres - k ? o.ckpt_every - due : nres - k;
+      if (n < kResMinSteps) break;
+      const int f1 = scratch_index(st, -1), f2 = scratch_index(st, f1);
+      void* const uu[2] = {st->buf[st->cur], res32 ? st->buf[f1] : nullptr};
+      void* const vv[2] = {st->buf[st->aux], res32 ? st->buf[f2] : nullptr};
+      void* tr = o.traces ? (char*)o.traces + (size_t)k * o.nrec * elem_size(dtype) : nullptr;
+      double* en = o.energy ? o.energy + k : nullptr;
+      cudaError_t e = cudaSuccess;
+      if (o.ckpt && due == 0 && (res32 ? tsu::res_fits(sg, o.energy != nullptr) : tsu::res64_fits(sg, ews)))
+        e = checkpoint(st, o, field_bytes, s);
+      int last = 0;
+      if (e == cudaSuccess)
+        e = res32 ? tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, en, ews, n, s, o.nrec, o.rec_idx, tr, k == 0, &ran,
+                                         &last)
+                  : tsu::launch_step_res64(sg, m->hx, m->hy, uu[0], vv[0], en, ews, n, s, o.nrec, o.rec_idx, tr, &ran);
+      if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n resident launch");
+      if (!ran) break;
       if (last == 1) {
         st->cur = f1;
         st->aux = f2;
       }
-      st->step += nres;
-      k = nres;
+      st->step += n;
+      k += n;
     }
   }
-  if (o.kernel == 0 && o.rows == 0 && dtype == TSU_F64 && st->form == TSU_FORM_STANDARD && have_ws && !o.ckpt &&
-      nsteps >= kResMinSteps && (!o.traces || o.nrec <= tsu::kResMaxRec)) {
-    bool ran = false;
-    cudaError_t e = tsu::launch_step_res64(sg, m->hx, m->hy, st->buf[st->cur], st->buf[st->aux], o.energy, ews, nsteps,
-                                           s, o.nrec, o.rec_idx, o.traces, &ran);
-    if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n resident FP64 launch");
-    if (ran) {
-      st->step += nsteps;
-      return TSU_OK;
-    }
-  }
-  if (k == 0 && use_wtb && o.traces) {
+  if (use_wtb && o.traces && k + wdepth <= nsteps) {
     cudaError_t e = tsu::launch_wtb_rec_table(sg, wrows, o.rec_idx, o.nrec, ews, s);
-    if (e == cudaSuccess) e = tsu::launch_wtb_trace_edges(sg, o.rec_idx, o.nrec, o.traces, nsteps / wdepth * wdepth, s);
+    if (e == cudaSuccess)
+      e = tsu::launch_wtb_trace_edges(sg, o.rec_idx, o.nrec, (float*)o.traces + k * o.nrec,
+                                      (nsteps - k) / wdepth * wdepth, s);
     if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n receiver table");
   }
   if (k == 0 && use_wtb && flow_possible && (o.kernel == 4 || (o.kernel == 0 && tsu::wtb_flow_preferred(g->ny, g->ld)))) {
@@ -440,12 +455,8 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   if (use_wtb) {
     for (; k + wdepth <= nsteps; k += wdepth) {
       const int64_t n = st->step;  // state holds u^n: checkpoint (u^{n-1}, u^n) or (u^n, v^n)
-      if (o.ckpt && ((n - 1) % o.ckpt_every) == 0 && (n - 1) / o.ckpt_every < o.ckpt_slots) {
-        char* slot = (char*)o.ckpt + (size_t)((n - 1) / o.ckpt_every) * 2 * field_bytes;
-        const void* a0 = st->form == TSU_FORM_STANDARD ? st->buf[st->aux] : st->buf[st->cur];
-        const void* a1 = st->form == TSU_FORM_STANDARD ? st->buf[st->cur] : st->buf[st->aux];
-        cudaError_t e = cudaMemcpyAsync(slot, a0, field_bytes, cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(slot + field_bytes, a1, field_bytes, cudaMemcpyDeviceToDevice, s);
+      if (o.ckpt && ((n - 1) % o.ckpt_every) == 0) {
+        cudaError_t e = checkpoint(st, o, field_bytes, s);
         if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n checkpoint");
       }
       const int f1 = scratch_index(st, -1), f2 = scratch_index(st, f1);

@@ -62,11 +62,13 @@ constexpr int kResMaxCtas = 160;
 constexpr int32_t kResMaxRec = 512;  // receivers a CTA keeps in its list
 size_t res_bytes(int64_t ny, int64_t ld);  // 0: the grid does not fit
 // nsteps steps (FP32, increment form): from (u, v)[0], using (u, v)[1] as the other pair;
-// the state ends up in (u, v)[*last].  energy and traces per step, or nullptr.  *ran = false and
+// the state ends up in (u, v)[*last].  table: build the receiver table (the first launch of a call).
+//   energy and traces per step, or nullptr.  *ran = false and
 // nothing enqueued when the device, the workspace or the grid do not allow it.
 cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
                             double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
-                            const int64_t* rec_idx, void* traces, bool* ran, int* last);
+                            const int64_t* rec_idx, void* traces, bool table, bool* ran, int* last);
+bool res_fits(const StencilGeom& g, bool energy);  // on this device
 
 // The same for FP64 grids of up to about 750^2 in the standard form (k_step_res64.cu): u = u^n and
 // p = u^{n-1} are updated in place.
@@ -74,6 +76,7 @@ size_t res64_bytes(int64_t ny, int64_t ld);
 cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* hy, void* u, void* p, double* energy,
                               const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
                               const int64_t* rec_idx, void* traces, bool* ran);
+bool res64_fits(const StencilGeom& g, const EnergyWs& ews);
 
 // receivers the warp-blocked pass records itself (longer lists go one step per pass)
 constexpr int32_t kWtbMaxReceivers = 2048;
