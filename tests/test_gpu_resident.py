@@ -109,3 +109,29 @@ def test_capture_and_side_stream():
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(sim.u, ref)
+
+
+@pytest.mark.parametrize("dtype,nx,ny", [("f32", 300, 200), ("f32", 1025, 900), ("f64", 129, 257)])
+@pytest.mark.parametrize("every,calls", [(16, (70, 21)), (10, (47, 30)), (5, (23,)), (64, (64, 64, 9))])
+def test_checkpoints(dtype, nx, ny, every, calls):
+    """A launch per stretch between checkpoints: the same checkpoints, states and traces as one step per
+    pass, also when a call starts or ends between two, and when a stretch is too short for a launch."""
+    out = []
+    for kernel in (0, 1):
+        sim = tsu.Simulation.create(nx, DEPTH, dtype=dtype, ny=ny)
+        rng = np.random.default_rng(3)
+        u0 = tsu.empty_field(sim.g, dtype)
+        u0[1:-1, 1 : nx - 1] = torch.from_numpy(rng.standard_normal((ny - 2, nx - 2))).to(u0.dtype).cuda()
+        rec = torch.from_numpy(rng.integers(0, ny * sim.g.ld, 9)).cuda()
+        sim.init(u0)
+        ck = torch.full((sum(calls) // every + 2, 2, sim.g.ny, sim.g.ld), 5.0, dtype=u0.dtype, device="cuda")
+        tr = torch.zeros((sum(calls), 9), dtype=u0.dtype, device="cuda")
+        at = 0
+        for n in calls:
+            sim.step(n, ckpt=ck, ckpt_every=every, rec_idx=rec, traces=tr[at : at + n], kernel=kernel)
+            at += n
+        torch.cuda.synchronize()
+        other = sim.v if sim.form == tsu.TSU_FORM_INCREMENT else sim.u_prev
+        out.append((sim.u.clone(), other.clone(), ck, tr))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
