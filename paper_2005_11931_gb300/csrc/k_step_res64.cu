@@ -52,6 +52,8 @@ struct R64Args {
   double* traces;
   int32_t nrec;
   const int64_t* rec_idx;
+  double* seg;  // or nullptr: u^{n+1+k} into seg + k seg_stride, and u, p left as they are
+  int64_t seg_stride;
 };
 
 __device__ __forceinline__ void put64(uint4* d, const double x, const uint32_t tag) {
@@ -80,6 +82,7 @@ __device__ __forceinline__ double get64(uint4 x, const uint4* d, const uint32_t 
     }
     dead = it >= kSpinCap;
   }
+  if (dead) return __longlong_as_double(0x7ff8000000000000ll);  // a wait ran out: nothing that follows is valid
   return __longlong_as_double((long long)((unsigned long long)x.z << 32 | x.x));
 }
 
@@ -189,6 +192,12 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_leapfrog_res64(const R64Args
       gd = gu;
     }
     if constexpr (ENERGY) sm.es[n & (kR64Sum - 1)][tid] = node ? e : 0.0;
+    if (a.seg && node) {
+      double* d = a.seg + (int64_t)n * a.seg_stride + (int64_t)j0 * a.ld + c;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (r < cnt) d[(int64_t)r * a.ld] = u[r];
+    }
     const bool last = n + 1 == (int)a.nsteps;
     if (!last) {
       const int q = n & 1;
@@ -250,7 +259,7 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_leapfrog_res64(const R64Args
       }
     }
   }
-  if (node) {
+  if (node && !a.seg) {
 #pragma unroll
     for (int r = 0; r < R; ++r)
       if (r < cnt) {
@@ -258,7 +267,7 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_leapfrog_res64(const R64Args
         a.p[(int64_t)(j0 + r) * a.ld + c] = p[r];
       }
   }
-  if (dead) atomicExch(a.status, (int)TSU_ETIMEOUT);
+  if (dead && a.status) atomicExch(a.status, (int)TSU_ETIMEOUT);
 }
 
 using R64Kernel = void (*)(const R64Args);
@@ -311,30 +320,26 @@ size_t res64_bytes(int64_t ny, int64_t ld) {
 }
 
 // The variant and the rows per CTA (one CTA per SM, as many as fit); -1: the grid does not fit.
-static int r64_plan(const StencilGeom& g, const EnergyWs& ews, int64_t* rows) {
+static int r64_plan(const StencilGeom& g, int64_t* rows) {
   const int64_t sms = r64_sms(), strips = r64_strips(g.nx), inner = g.ny - 2;
-  if (sms <= 0 || strips < 1 || strips > sms || !ews.res || !ews.status || g.ny >= 1 << 22 ||
-      ews.res_size < kR64RimBytes + (size_t)kR64EnergySteps * kResMaxCtas * sizeof(double))
-    return -1;
+  if (sms <= 0 || strips < 1 || strips > sms || g.ny >= 1 << 22) return -1;
   *rows = (inner + sms / strips - 1) / (sms / strips);
   const int64_t per_warp = (*rows + kR64Warps - 1) / kR64Warps;
   for (int k = 0; k < kR64Num; ++k)
     if (kR64Variants[k].rows >= per_warp) return k;
   return -1;
 }
+static bool r64_workspace(const EnergyWs& ews) {
+  return ews.res && ews.status &&
+         ews.res_size >= kR64RimBytes + (size_t)kR64EnergySteps * kResMaxCtas * sizeof(double);
+}
 bool res64_fits(const StencilGeom& g, const EnergyWs& ews) {
   int64_t rows = 0;
-  return r64_plan(g, ews, &rows) >= 0;
+  return r64_workspace(ews) && r64_plan(g, &rows) >= 0;
 }
 
-cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* hy, void* u, void* p, double* energy,
-                              const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
-                              const int64_t* rec_idx, void* traces, bool* ran) {
-  *ran = false;
-  int64_t rows = 0;
-  const int k = r64_plan(g, ews, &rows);
-  if (k < 0 || nsteps >= 1ll << 31 || (traces && nrec > kResMaxRec)) return cudaSuccess;
-  const int64_t strips = r64_strips(g.nx), inner = g.ny - 2;
+static R64Args r64_args(const StencilGeom& g, const void* hx, const void* hy, const void* u, const void* p, int64_t rows,
+                        void* rims) {
   R64Args a{};
   a.nx = g.nx;
   a.ny = g.ny;
@@ -346,17 +351,19 @@ cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* 
   a.u = (double*)u;
   a.p = (double*)p;
   a.rows = (int)rows;
-  a.nstrips = (int)strips;
-  a.nchunks = (int)((inner + rows - 1) / rows);
-  const int ncta = a.nstrips * a.nchunks;
-  a.col = (uint4*)ews.res;
-  a.row = a.col + (int64_t)2 * ncta * 2 * kR64Rows;
-  a.part = (double*)((char*)ews.res + kR64RimBytes);
-  a.status = ews.status;
-  a.nrec = traces ? nrec : 0;
-  a.rec_idx = rec_idx;
+  a.nstrips = (int)r64_strips(g.nx);
+  a.nchunks = (int)((g.ny - 2 + rows - 1) / rows);
+  a.col = (uint4*)rims;
+  a.row = a.col + (int64_t)2 * a.nstrips * a.nchunks * 2 * kR64Rows;
+  return a;
+}
+
+static cudaError_t r64_launch(const R64Args& a, R64Kernel kern, cudaStream_t s) {
+  // no value may carry a tag of an earlier launch
+  const cudaError_t e = cudaMemsetAsync(a.col, 0, kR64RimBytes, s);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)ncta);
+  cfg.gridDim = dim3((unsigned)(a.nstrips * a.nchunks));
   cfg.blockDim = dim3(kR64Threads);
   cfg.dynamicSmemBytes = sizeof(R64Smem);
   cfg.stream = s;
@@ -365,18 +372,51 @@ cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* 
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* hy, void* u, void* p, double* energy,
+                              const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
+                              const int64_t* rec_idx, void* traces, bool* ran) {
+  *ran = false;
+  int64_t rows = 0;
+  const int k = r64_workspace(ews) ? r64_plan(g, &rows) : -1;
+  if (k < 0 || nsteps >= 1ll << 31 || (traces && nrec > kResMaxRec)) return cudaSuccess;
+  R64Args a = r64_args(g, hx, hy, u, p, rows, ews.res);
+  a.part = (double*)((char*)ews.res + kR64RimBytes);
+  a.status = ews.status;
+  a.nrec = traces ? nrec : 0;
+  a.rec_idx = rec_idx;
   for (int64_t n = 0; n < nsteps; n += a.nsteps) {
     a.nsteps = energy && nsteps - n > kR64EnergySteps ? kR64EnergySteps : nsteps - n;
     if (nsteps - n - a.nsteps == 1) a.nsteps -= 1;  // no launch of a single step (it writes in place)
     a.traces = traces ? (double*)traces + n * nrec : nullptr;
-    // no value may carry a tag of an earlier launch
-    cudaError_t e = cudaMemsetAsync(ews.res, 0, kR64RimBytes, s);
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kR64Variants[k].kern[energy ? 1 : 0], a);
-    if (e == cudaSuccess && energy) e = launch_energy64(g, a.part, ncta, a.nsteps, energy + n, s);
+    cudaError_t e = r64_launch(a, kR64Variants[k].kern[energy ? 1 : 0], s);
+    if (e == cudaSuccess && energy)
+      e = launch_energy64(g, a.part, (int64_t)a.nstrips * a.nchunks, a.nsteps, energy + n, s);
     if (e != cudaSuccess) return e;
   }
   *ran = true;
   return cudaSuccess;
+}
+
+size_t res64_seg_bytes(const StencilGeom& g) {
+  return r64_strips(g.nx) * ((g.ny - 2 + kR64Rows - 1) / kR64Rows) <= kResMaxCtas ? kR64RimBytes : 0;
+}
+
+cudaError_t launch_step_res64_seg(const StencilGeom& g, const void* hx, const void* hy, const void* u, const void* p,
+                                  void* seg, int64_t seg_stride, int64_t nsteps, void* ws, cudaStream_t s, bool* ran) {
+  *ran = false;
+  int64_t rows = 0;
+  const int k = ws ? r64_plan(g, &rows) : -1;
+  if (k < 0 || nsteps < 1 || nsteps >= 1ll << 31) return cudaSuccess;
+  R64Args a = r64_args(g, hx, hy, u, p, rows, ws);
+  a.nsteps = nsteps;
+  a.seg = (double*)seg;
+  a.seg_stride = seg_stride;
+  const cudaError_t e = r64_launch(a, kR64Variants[k].kern[0], s);
+  *ran = e == cudaSuccess;
+  return e;
 }
 
 }  // namespace tsu

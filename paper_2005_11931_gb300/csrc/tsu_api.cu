@@ -568,6 +568,7 @@ static size_t adjoint_ws_bytes(const tsu_grid* g, int dtype, int form, int64_t e
   size_t b = (size_t)adjoint_fields(form, every) * fb;
   if (dtype == TSU_F32) b += 2 * (size_t)g->ny * g->ld * sizeof(float);
   const size_t buckets = adjoint_bucket_bytes(g, dtype, nrec);
+  if (dtype == TSU_F64) b += 256 + tsu::res64_seg_bytes(geom(g, 1.0));  // the recompute on chip
   return b + (buckets + 255) / 256 * 256 + 256;
 }
 
@@ -707,6 +708,9 @@ int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_me
   auto segp = [&](int b, int64_t k) { return (void*)(segbuf[b] + (size_t)k * fb); };
   const int recompute_rows = tsu::wtb_seg_rows(g->ny, g->ld);
   auto extra = [&](int b, int q = 0) { return (void*)(segbuf[b] + (size_t)(ckpt_every + 1 + q) * fb); };
+  void* res_ws = nullptr;  // FP64: the last part of the workspace
+  if (dtype == TSU_F64 && tsu::res64_seg_bytes(sg))
+    res_ws = (void*)(((uintptr_t)w + need - 256 - tsu::res64_seg_bytes(sg)) / 128 * 128);
   AuxStream* aux = aux_stream();
   if (!aux) return fail(TSU_ECUDA, "tsu_adjoint: could not create the recompute stream");
   cudaError_t e = cudaMemsetAsync(ws, 0, need - 256, s);
@@ -793,6 +797,13 @@ int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_me
         if (e != cudaSuccess) return cuda_fail(e, "tsu_adjoint recompute");
         vq ^= 1;
       }
+    }
+    if (dtype == TSU_F64 && form == TSU_FORM_STANDARD && mend - mc >= kResMinSteps) {
+      bool ran = false;  // the whole segment in one launch where the grid fits on chip
+      e = tsu::launch_step_res64_seg(sg, m->hx, m->hy, segp(b, 0), extra(b), segp(b, 1), (int64_t)(fb / es), mend - mc,
+                                     res_ws, aux->s, &ran);
+      if (e != cudaSuccess) return cuda_fail(e, "tsu_adjoint recompute");
+      if (ran) k = mend - mc;
     }
     for (; k < mend - mc; ++k) {
       if (form == TSU_FORM_STANDARD)

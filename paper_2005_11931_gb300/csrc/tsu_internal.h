@@ -77,6 +77,11 @@ cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* 
                               const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
                               const int64_t* rec_idx, void* traces, bool* ran);
 bool res64_fits(const StencilGeom& g, const EnergyWs& ews);
+// the same storing every state, u^{n+1+k} into seg + k seg_stride (elements), u = u^n and p = u^{n-1} left
+// as they are; ws: res64_seg_bytes(g) bytes (0: the grid does not fit).  A wait that ran out leaves NaN.
+size_t res64_seg_bytes(const StencilGeom& g);
+cudaError_t launch_step_res64_seg(const StencilGeom& g, const void* hx, const void* hy, const void* u, const void* p,
+                                  void* seg, int64_t seg_stride, int64_t nsteps, void* ws, cudaStream_t s, bool* ran);
 
 // receivers the warp-blocked pass records itself (longer lists go one step per pass)
 constexpr int32_t kWtbMaxReceivers = 2048;
