@@ -17,7 +17,7 @@
 // windows, as k_step_wtb.cu does, takes 100 to 176), and one exchange, about 2 us, per four steps.
 // Measured (GB300, us per step, before and after): 769^2 with receivers 4.1 and 1.35; 1024^2 3.6 and
 // 1.43, 1400^2 4.6 and 1.9, 2048^2 5.9 and 4.7; with the energy 1003 x 517 4.8 and 1.7, 1024^2 4.9 and
-// 2.0, 1536^2 5.7 and 3.0.
+// 2.0, 1536^2 5.7 and 3.0, 2048^2 6.85 and 6.05.
 //
 // All warps run the row code in step (a barrier per step): when only neighbouring warps waited for
 // each other they drifted apart, and the unrolled code of all of them no longer fitted the
@@ -77,6 +77,7 @@ struct ResArgs {
   int rows, nstrips, nchunks;
   int64_t nsteps;
   double* part;  // [step][CTA] energy partials
+  float2* es;    // [CTA][kResK][thread], lean tiles
   ResItem* col;  // [2][CTA][2][16 R] the first and last output lane of every row
   ResItem* row;  // [2][CTA][2][4][32] the first and last four output rows
   int* status;
@@ -88,17 +89,23 @@ struct ResArgs {
 
 // rows r < kTmemRows of a wide tile keep their faces in tensor memory
 constexpr int kTmemRows = 16;
+// Wide tiles of more than 12 rows with the energy: shared memory holds the terms of one step only (a
+// barrier more per step, between the chains and the next rows), the rims' staging shares their
+// place, and the chains' results of a pass wait in the workspace.
+constexpr bool res_lean(int R, bool ENERGY) { return ENERGY && R > 12; }
 template <int R, bool WIDE, bool ENERGY>
 struct ResSmem {
+  static constexpr bool kLean = res_lean(R, ENERGY);
+  static constexpr int kStage = 4 * R > 32 ? 4 * R : 32;
   float4 xch[2][kResWarps][2][32];   // first and last u row of every warp, double buffered
   // energy: the terms of the last two steps summed over each lane's columns, the (sum, error) of each
   // thread's chain of rows for the pass's steps, and those of each warp
-  float er[ENERGY ? 2 : 1][ENERGY ? kResWarps * R : 1][32];
-  float2 es[ENERGY ? kResK : 1][kResThreads];
+  alignas(16) float er[ENERGY && !kLean ? 2 : 1][ENERGY ? kResWarps * R : 1][32];
+  float2 es[ENERGY && !kLean ? kResK : 1][ENERGY && !kLean ? kResThreads : 1];
   float2 esw[kResK][kResWarps];
   int2 rec[kResMaxRec];              // (row << 8 | column in the tile, receiver)
   // per warp: one row of u, or the values of its first and last output lanes on their way
-  float4 stage[kResWarps][4 * R > 32 ? 4 * R : 32];
+  float4 stage[kLean ? 1 : kResWarps][kLean ? 1 : kStage];
   uint32_t tmem;
   // narrow: [R][2] float4 per thread (hx, hy); wide: [R] v, the faces of the rows past kTmemRows
   // or else the hy row below the warp's first
@@ -191,6 +198,9 @@ __device__ __forceinline__ void pair_add(float2& a, const float2 b) {
 template <int R, int RB, bool WIDE, bool ENERGY, bool REC>
 __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a) {
   using Smem = ResSmem<R, WIDE, ENERGY>;
+  constexpr bool LEAN = Smem::kLean;
+  static_assert(!LEAN || !REC, "no place to stage receivers");
+  static_assert(!LEAN || sizeof(Smem::er) >= sizeof(float4) * kResWarps * Smem::kStage, "staging");
   extern __shared__ __align__(16) unsigned char res_raw[];
   Smem& sm = *reinterpret_cast<Smem*>(res_raw);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -254,6 +264,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
     const bool ok = col_in && rw - 1 >= 0 && rw - 1 < a.ny && rw - 1 < y1 + kResK;
     sm.f[Smem::kField - 1][tid] = ldcg4(a.hy + goff(-1), ok);
   }
+  float4* const stage = (LEAN ? reinterpret_cast<float4*>(&sm.er[0][0][0]) : &sm.stage[0][0]) + w * Smem::kStage;
   // receivers of the tile's own nodes; rec_rows: this warp's rows that hold some
   [[maybe_unused]] int nrec = 0;
   [[maybe_unused]] uint32_t rec_rows = 0;
@@ -327,13 +338,16 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
     if (col_out) {
 #pragma unroll 4
       for (int r = r0; r < r1; ++r) {
-        const float y = sm.er[s & 1][r][lane] - ec;
+        const float y = sm.er[LEAN ? 0 : s & 1][r][lane] - ec;
         const float sum = es + y;
         ec = (sum - es) - y;
         es = sum;
       }
     }
-    sm.es[s][tid] = make_float2(es, -ec);
+    if constexpr (LEAN)
+      a.es[((int64_t)cta * kResK + s) * kResThreads + tid] = make_float2(es, -ec);
+    else
+      sm.es[s][tid] = make_float2(es, -ec);
   };
 
   int buf = 0;
@@ -353,7 +367,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       const P4 above = w + 1 < kResWarps ? as_p4(sm.xch[buf][w + 1][0][lane]) : zero;
       buf ^= 1;
       if constexpr (ENERGY) {
-        if (s > 0) chain(s - 1);
+        if (s > 0) {
+          chain(s - 1);
+          if constexpr (LEAN) __syncthreads();
+        }
       }
       {
         P4 gb;  // y flux below the current row
@@ -420,13 +437,13 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
             if (r >= R) continue;
             if constexpr (REC) {
               if ((rec_rows >> r) & 1u) {  // receivers on this row: u^{n} before the step
-                sm.stage[w][lane] = as_f4(u[r]);
+                stage[lane] = as_f4(u[r]);
                 __syncwarp();
                 for (int q = lane; q < nrec; q += 32) {
                   const int2 e = sm.rec[q];
                   if ((e.x >> 8) == rw + r)
                     a.traces[((int64_t)p * kResK + s) * a.nrec + e.y] =
-                        reinterpret_cast<const float*>(sm.stage[w])[e.x & 255];
+                        reinterpret_cast<const float*>(stage)[e.x & 255];
                 }
                 __syncwarp();
               }
@@ -451,7 +468,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
               u[r].p[q] = add2(u[r].p[q], vn.p[q]);
             }
             set_v(r, vn);
-            if constexpr (ENERGY) sm.er[s & 1][w * R + r][lane] = erow;
+            if constexpr (ENERGY) sm.er[LEAN ? 0 : s & 1][w * R + r][lane] = erow;
           }
           gb = gy[RB - 1];
         }
@@ -471,6 +488,11 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
     const bool last = p + 1 == npass;
     const int q = p & 1;
     const uint32_t tag = (uint32_t)p + 1u;
+    if constexpr (LEAN) {
+      __syncthreads();
+      chain(ns - 1);
+      __syncthreads();
+    }
     if (!last) {
       // ---- the rims: four rows (all output lanes) where this warp holds them, and its two output
       // columns of lanes, gathered in shared memory so that each lane sends one row's
@@ -487,14 +509,14 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       if (lx == 1 || lx == 30) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          sm.stage[w][4 * r + (lx == 30 ? 2 : 0)] = as_f4(u[r]);
-          sm.stage[w][4 * r + (lx == 30 ? 3 : 1)] = as_f4(get_v(r));
+          stage[4 * r + (lx == 30 ? 2 : 0)] = as_f4(u[r]);
+          stage[4 * r + (lx == 30 ? 3 : 1)] = as_f4(get_v(r));
         }
       }
       __syncwarp();
       for (int k = lx; k < 2 * R; k += 32)
         if ((k & 1) ? has_r : has_l)
-          item_put(col_rim(q, cta, k & 1) + (k >> 1), sm.stage[w][2 * k], sm.stage[w][2 * k + 1], tag);
+          item_put(col_rim(q, cta, k & 1) + (k >> 1), stage[2 * k], stage[2 * k + 1], tag);
     } else if (col_out) {  // ---- the end: the whole tile
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -507,12 +529,17 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       }
     }
     if constexpr (ENERGY) {
-      __syncthreads();
-      chain(ns - 1);
+      if constexpr (!LEAN) {
+        __syncthreads();
+        chain(ns - 1);
+      }
       // the warp's sums of the pass's steps: lanes 8 t .. 8 t + 7 end up with step t
       float2 e[kResK];
 #pragma unroll
-      for (int t = 0; t < kResK; ++t) e[t] = t < ns ? sm.es[t][tx] : make_float2(0.f, 0.f);
+      for (int t = 0; t < kResK; ++t) {
+        e[t] = make_float2(0.f, 0.f);
+        if (t < ns) e[t] = LEAN ? a.es[((int64_t)cta * kResK + t) * kResThreads + tx] : sm.es[LEAN ? 0 : t][LEAN ? 0 : tx];
+      }
       auto fold = [&](float2& keep, const float2& send, int o) {
         pair_add(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, o), __shfl_xor_sync(0xffffffffu, send.y, o)));
       };
@@ -560,7 +587,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
         const int k = i - 16;
         if (((k & 1) ? has_r : has_l) && ((own_rows >> (k >> 1)) & 1u)) {
           src = col_rim(q, (k & 1) ? cta + 1 : cta - 1, (k & 1) ^ 1) + (k >> 1);
-          dst = &sm.stage[w][2 * k];
+          dst = &stage[2 * k];
         }
       }
       if (src) {
@@ -575,8 +602,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         if (!((own_rows >> r) & 1u)) continue;
-        u[r] = as_p4(sm.stage[w][4 * r + (lx == 31 ? 2 : 0)]);
-        set_v(r, as_p4(sm.stage[w][4 * r + (lx == 31 ? 3 : 1)]));
+        u[r] = as_p4(stage[4 * r + (lx == 31 ? 2 : 0)]);
+        set_v(r, as_p4(stage[4 * r + (lx == 31 ? 3 : 1)]));
       }
     }
     __syncthreads();  // halo complete; the energy slots are free again
@@ -619,8 +646,10 @@ struct ResVariant {
 };
 template <int R, int RB, bool WIDE, bool ENERGY>
 constexpr ResVariant res_variant() {
-  return ResVariant{R, sizeof(ResSmem<R, WIDE, ENERGY>),
-                    {k_leapfrog_res<R, RB, WIDE, ENERGY, false>, k_leapfrog_res<R, RB, WIDE, ENERGY, true>}};
+  static_assert(sizeof(ResSmem<R, WIDE, ENERGY>) <= 227 * 1024, "shared memory of a CTA");
+  ResVariant v{R, sizeof(ResSmem<R, WIDE, ENERGY>), {k_leapfrog_res<R, RB, WIDE, ENERGY, false>, nullptr}};
+  if constexpr (!res_lean(R, ENERGY)) v.kern[1] = k_leapfrog_res<R, RB, WIDE, ENERGY, true>;
+  return v;
 }
 // without the energy, then with it
 const ResVariant kResVariants[] = {
@@ -630,7 +659,7 @@ const ResVariant kResVariants[] = {
     res_variant<14, 2, true, false>(),  res_variant<17, 2, true, false>(), res_variant<2, 2, false, true>(),
     res_variant<3, 3, false, true>(),   res_variant<4, 2, false, true>(),  res_variant<5, 2, true, true>(),
     res_variant<6, 2, true, true>(),   res_variant<8, 2, true, true>(),  res_variant<10, 2, true, true>(),
-    res_variant<12, 2, true, true>()};
+    res_variant<12, 2, true, true>(),   res_variant<14, 2, true, true>(),  res_variant<17, 2, true, true>()};
 constexpr int kResPlain = 11;  // variants without the energy
 constexpr int kResNumVariants = (int)(sizeof kResVariants / sizeof kResVariants[0]);
 // own rows of a tile: with the energy whole chains
@@ -652,6 +681,7 @@ int res_sms() {
   for (int k = 0; ok && k < 2 * kResNumVariants; ++k) {
     const ResVariant& x = kResVariants[k / 2];
     int q = 0;
+    if (!x.kern[k & 1]) continue;
     ok = cudaFuncSetAttribute(x.kern[k & 1], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)x.smem) ==
              cudaSuccess &&
          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, x.kern[k & 1], kResThreads, x.smem) == cudaSuccess &&
@@ -672,14 +702,17 @@ int64_t res_strips(int64_t ld) { return (ld + 4 + kResOut - 1) / kResOut; }
 static size_t res_rim_bytes(int k, int64_t ncta) {
   return (size_t)ncta * 2 * (2 * kResWarps * kResVariants[k].rows + 2 * kResK * 32) * sizeof(ResItem);
 }
-static size_t res_part_bytes(int64_t ncta) { return (size_t)kResEnergySteps * ncta * sizeof(double); }
+static size_t res_part_bytes(int k, int64_t ncta) {
+  const bool lean = res_lean(kResVariants[k].rows, k >= kResPlain);
+  return (size_t)ncta * (kResEnergySteps * sizeof(double) + (lean ? kResK * kResThreads * sizeof(float2) : 0));
+}
 size_t res_bytes(int64_t ny, int64_t ld) {
   size_t most = 0;
   for (int k = 0; k < kResNumVariants; ++k) {
     const int64_t cap = res_cap(k);
     const int64_t ncta = res_strips(ld) * ((ny - 2 + cap - 1) / cap);
     if (ncta > kResMaxCtas) continue;
-    const size_t b = res_rim_bytes(k, ncta) + res_part_bytes(ncta);
+    const size_t b = res_rim_bytes(k, ncta) + (k < kResPlain ? 0 : res_part_bytes(k, ncta));
     if (b > most) most = b;
   }
   return most;
@@ -733,10 +766,12 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
   a.nstrips = (int)res_strips(g.ld);
   a.nchunks = (g.ny - 2 + rows - 1) / rows;
   const ResVariant& x = kResVariants[k];
+  if (!x.kern[traces && nrec > 0 ? 1 : 0]) return cudaSuccess;
   const int64_t ncta = (int64_t)a.nstrips * a.nchunks;
   a.col = (ResItem*)ews.res;
   a.row = a.col + 2 * ncta * 2 * kResWarps * x.rows;
   a.part = (double*)((char*)ews.res + res_rim_bytes(k, ncta));
+  a.es = (float2*)(a.part + kResEnergySteps * ncta);
   a.status = ews.status;
   cudaError_t e = cudaSuccess;
   if (traces && nrec > 0) {
