@@ -54,7 +54,10 @@ constexpr int kResOut = 120;    // output columns per strip: strip s reads 120 s
 // on chip and writes them back, about 15 us for 1024 steps of 1 ms or more).
 constexpr int64_t kResEnergySteps = 1024;
 constexpr int kResChain = 16;  // rows of an energy chain (k_step_wtb.cu's smallest tile)
-constexpr uint64_t kResWaitNs = 2000000000ull;
+// A launch never runs longer than a fraction of a second, so that another resident launch on the
+// device, whose CTAs may be placed as this one's leave, gets its SMs well inside the bound of its waits.
+constexpr int64_t kResMaxSteps = 16384;
+constexpr uint64_t kResWaitNs = 10000000000ull;
 
 // One lane's four columns of u and v as they travel between CTAs: every 8 bytes hold a value and
 // the number of the pass that wrote it, so a reader polls the data itself and no flag, fence or
@@ -793,7 +796,8 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
   cfg.attrs = at;
   cfg.numAttrs = 1;
   for (int64_t n = 0; n < nsteps; n += a.nsteps) {
-    a.nsteps = energy && nsteps - n > kResEnergySteps ? kResEnergySteps : nsteps - n;
+    const int64_t most = energy ? kResEnergySteps : kResMaxSteps;
+    a.nsteps = nsteps - n > most ? most : nsteps - n;
     a.u = (const float*)u[*last];
     a.v = (const float*)v[*last];
     *last ^= 1;

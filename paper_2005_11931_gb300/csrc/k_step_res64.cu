@@ -20,20 +20,17 @@
 // lanes of step t, which costs one FP64 instruction per warp and step instead of a shuffle tree's five.
 #include <atomic>
 
-#include "async_copy.cuh"
+#include "resident64.cuh"
 #include "stencil_common.cuh"
 
 namespace tsu {
 namespace {
 using namespace dev;
 
-constexpr int kR64Warps = 8, kR64Threads = kR64Warps * 32;
-constexpr int kR64Out = 30;             // own columns of a strip: 30 s + 1 .. 30 s + 30
-constexpr int kR64MaxRows = 16;         // rows per warp
-constexpr int kR64Rows = kR64Warps * kR64MaxRows;
-constexpr int kR64Sum = 32;             // steps whose energy terms are summed together
+constexpr int kR64MaxRows = 16;           // rows per warp
+constexpr int kR64Sum = 32;               // steps whose energy terms are summed together
+constexpr int64_t kR64MaxSteps = 16384;   // steps per launch (a fraction of a second: see k_step_res.cu)
 constexpr int64_t kR64EnergySteps = 512;  // steps per launch with the energy (partials kept)
-constexpr uint64_t kR64WaitNs = 2000000000ull;
 
 struct R64Args {
   int32_t nx, ny;
@@ -55,36 +52,6 @@ struct R64Args {
   double* seg;  // or nullptr: u^{n+1+k} into seg + k seg_stride, and u, p left as they are
   int64_t seg_stride;
 };
-
-__device__ __forceinline__ void put64(uint4* d, const double x, const uint32_t tag) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %2};" ::"l"(d), "r"((uint32_t)b), "r"(tag),
-               "r"((uint32_t)(b >> 32))
-               : "memory");
-}
-__device__ __forceinline__ uint4 try64(const uint4* d) {
-  uint4 x;
-  asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w)
-               : "l"(d)
-               : "memory");
-  return x;
-}
-// the value of x, read again until both its halves carry the tag (bounded)
-__device__ __forceinline__ double get64(uint4 x, const uint4* d, const uint32_t tag, bool& dead) {
-  if (!(x.y == tag && x.w == tag) && !dead) {
-    const uint64_t t0 = global_ns();
-    long long it = 0;
-    for (; it < kSpinCap; ++it) {
-      x = try64(d);
-      if (x.y == tag && x.w == tag) break;
-      if ((it & 63) == 63 && global_ns() - t0 > kR64WaitNs) it = kSpinCap;
-    }
-    dead = it >= kSpinCap;
-  }
-  if (dead) return __longlong_as_double(0x7ff8000000000000ll);  // a wait ran out: nothing that follows is valid
-  return __longlong_as_double((long long)((unsigned long long)x.z << 32 | x.x));
-}
 
 struct R64Smem {
   double xch[2][kR64Warps][2][32];  // first and last row of every warp, double buffered
@@ -308,8 +275,7 @@ int r64_sms() {
   return v > 0 ? v : 0;
 }
 
-constexpr size_t kR64RimBytes = (size_t)2 * kResMaxCtas * 2 * (kR64Rows + 32) * sizeof(uint4);
-int64_t r64_strips(int64_t nx) { return (nx - 2 + kR64Out - 1) / kR64Out; }
+static_assert(kR64Warps * kR64MaxRows <= kR64Rows, "rows of a rim");
 
 }  // namespace
 
@@ -388,7 +354,8 @@ cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* 
   a.nrec = traces ? nrec : 0;
   a.rec_idx = rec_idx;
   for (int64_t n = 0; n < nsteps; n += a.nsteps) {
-    a.nsteps = energy && nsteps - n > kR64EnergySteps ? kR64EnergySteps : nsteps - n;
+    const int64_t most = energy ? kR64EnergySteps : kR64MaxSteps;
+    a.nsteps = nsteps - n > most ? most : nsteps - n;
     if (nsteps - n - a.nsteps == 1) a.nsteps -= 1;  // no launch of a single step (it writes in place)
     a.traces = traces ? (double*)traces + n * nrec : nullptr;
     cudaError_t e = r64_launch(a, kR64Variants[k].kern[energy ? 1 : 0], s);
@@ -409,7 +376,7 @@ cudaError_t launch_step_res64_seg(const StencilGeom& g, const void* hx, const vo
   *ran = false;
   int64_t rows = 0;
   const int k = ws ? r64_plan(g, &rows) : -1;
-  if (k < 0 || nsteps < 1 || nsteps >= 1ll << 31) return cudaSuccess;
+  if (k < 0 || nsteps < 1 || nsteps > kR64MaxSteps) return cudaSuccess;
   R64Args a = r64_args(g, hx, hy, u, p, rows, ws);
   a.nsteps = nsteps;
   a.seg = (double*)seg;

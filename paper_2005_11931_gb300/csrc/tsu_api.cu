@@ -568,7 +568,7 @@ static size_t adjoint_ws_bytes(const tsu_grid* g, int dtype, int form, int64_t e
   size_t b = (size_t)adjoint_fields(form, every) * fb;
   if (dtype == TSU_F32) b += 2 * (size_t)g->ny * g->ld * sizeof(float);
   const size_t buckets = adjoint_bucket_bytes(g, dtype, nrec);
-  if (dtype == TSU_F64) b += 256 + tsu::res64_seg_bytes(geom(g, 1.0));  // the recompute on chip
+  if (dtype == TSU_F64) b += 256 + 2 * tsu::res64_seg_bytes(geom(g, 1.0));  // recompute and sweep on chip
   return b + (buckets + 255) / 256 * 256 + 256;
 }
 
@@ -708,9 +708,9 @@ int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_me
   auto segp = [&](int b, int64_t k) { return (void*)(segbuf[b] + (size_t)k * fb); };
   const int recompute_rows = tsu::wtb_seg_rows(g->ny, g->ld);
   auto extra = [&](int b, int q = 0) { return (void*)(segbuf[b] + (size_t)(ckpt_every + 1 + q) * fb); };
-  void* res_ws = nullptr;  // FP64: the last part of the workspace
-  if (dtype == TSU_F64 && tsu::res64_seg_bytes(sg))
-    res_ws = (void*)(((uintptr_t)w + need - 256 - tsu::res64_seg_bytes(sg)) / 128 * 128);
+  // FP64: the last part of the workspace, for the recompute and for the sweep on chip
+  const size_t res_b = dtype == TSU_F64 ? tsu::res64_seg_bytes(sg) : 0;
+  char* res_ws = res_b ? (char*)(((uintptr_t)w + need - 256 - 2 * res_b) / 128 * 128) : nullptr;
   AuxStream* aux = aux_stream();
   if (!aux) return fail(TSU_ECUDA, "tsu_adjoint: could not create the recompute stream");
   cudaError_t e = cudaMemsetAsync(ws, 0, need - 256, s);
@@ -819,7 +819,16 @@ int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_me
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, aux->computed[b], 0);
     if (e != cudaSuccess) return cuda_fail(e, "tsu_adjoint stream order");
     const int64_t nlo = (c == 0) ? 1 : mc + 1;
-    for (int64_t n = mend; n >= nlo;) {
+    int64_t n_first = mend;
+    if (dtype == TSU_F64 && mend - nlo + 1 >= kResMinSteps) {  // the whole segment in one launch where it fits
+      bool ran = false;
+      e = tsu::launch_adjoint_res64(sg, m->hx, m->hy, lam4[i1], lam4[i2], segp(b, mend - mc), (int64_t)(fb / es), accx,
+                                    accy, nrec, rec_idx, nrec > 0 ? (const char*)dtraces + (size_t)(mend - 1) * nrec * es : nullptr,
+                                    mend - nlo + 1, res_ws ? res_ws + res_b : nullptr, s, &ran);
+      if (e != cudaSuccess) return cuda_fail(e, "tsu_adjoint resident sweep");
+      if (ran) n_first = nlo - 1;
+    }
+    for (int64_t n = n_first; n >= nlo;) {
       if (blocked && n - (kAdjointDepth - 1) >= nlo) {
         const void* u[kAdjointDepth];
         for (int f = 0; f < kAdjointDepth; ++f) u[f] = segp(b, n - f - mc);

@@ -82,6 +82,12 @@ bool res64_fits(const StencilGeom& g, const EnergyWs& ews);
 size_t res64_seg_bytes(const StencilGeom& g);
 cudaError_t launch_step_res64_seg(const StencilGeom& g, const void* hx, const void* hy, const void* u, const void* p,
                                   void* seg, int64_t seg_stride, int64_t nsteps, void* ws, cudaStream_t s, bool* ran);
+// nsteps reverse steps (k_adjoint_res64.cu) from lam = lam^{n+1}, lam_pp = lam^{n+2} (in place) with u^{n-k} at
+// u - k ustride and the receivers' values of step k at gv - k nrec; ws: res64_seg_bytes(g) bytes of its own
+cudaError_t launch_adjoint_res64(const StencilGeom& g, const void* hx, const void* hy, void* lam, void* lam_pp,
+                                 const void* u, int64_t ustride, void* gx, void* gy, int32_t nrec,
+                                 const int64_t* rec_idx, const void* gv, int64_t nsteps, void* ws, cudaStream_t s,
+                                 bool* ran);
 
 // receivers the warp-blocked pass records itself (longer lists go one step per pass)
 constexpr int32_t kWtbMaxReceivers = 2048;

@@ -49,3 +49,24 @@ def test_long_calls(steps):
     a, b = (run(90, 100, (steps,), k, True, 3) for k in (0, 1))
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and torch.equal(a[3], b[3])
     assert torch.allclose(a[2], b[2], rtol=1e-11, atol=0)
+
+
+# the reverse sweep (k_adjoint_res64.cu) of a checkpoint segment on chip (20 steps) against one launch per
+# step (segments of 7): the same operations in the same order, so the same bits; receivers on the edges of
+# tiles, several on one node, and more than a tile's list holds
+@pytest.mark.parametrize("nx,ny,nrec", [(3, 3, 2), (31, 32, 9), (33, 600, 40), (63, 64, 200), (201, 180, 0), (257, 300, 512),
+                                        (400, 390, 30), (500, 499, 64), (520, 200, 513), (121, 2400, 25), (700, 690, 8)])
+def test_adjoint_on_chip(nx, ny, nrec):
+    from tests.test_gpu_adjoint import gpu_forward_adjoint
+
+    S = 47
+    rng = np.random.default_rng(nx)
+    u0, u1 = inputs.random_field(nx, ny, None, rng), inputs.random_field(nx, ny, None, rng)
+    rec = np.stack([rng.integers(0, nx, max(nrec, 1)), rng.integers(0, ny, max(nrec, 1))], 1)[:nrec]
+    if nrec > 4:
+        rec[:4] = [[1, 1], [nx - 2, ny - 2], [min(30, nx - 2), ny // 2], [min(30, nx - 2), ny // 2]]
+    dtr = rng.standard_normal((S, nrec))
+    a, _ = gpu_forward_adjoint(nx, ny, DEPTH, u0, u1, S, rec, dtr, "f64", tsu.TSU_FORM_STANDARD, 20)
+    b, _ = gpu_forward_adjoint(nx, ny, DEPTH, u0, u1, S, rec, dtr, "f64", tsu.TSU_FORM_STANDARD, 7)
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
