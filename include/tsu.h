@@ -150,12 +150,16 @@ typedef struct {
                        passes (tdepth 4, increment form, no traces or checkpoints) all in one
                        persistent launch, a tile's next pass starting once the tiles
                        around it finished the current one (its waits are bounded: TSU_ETIMEOUT
-                       through tsu_sync_status); auto picks kernel 4 where it can run and its tiles
-                       number between half and 6 times the device's resident warps (FP32 grids
+                       through tsu_sync_status); auto (with rows = 0) keeps grids that fit on chip there for
+                       the whole call, or up to the next checkpoint, in one cooperative launch (FP32
+                       in the increment form with nbuf = 4 up to about 2000^2, FP64 in the standard
+                       form up to about 750^2; a workspace, at most 512 receivers, at least 8 steps;
+                       its waits are bounded as kernel 4's); else kernel 4 where it can run and its
+                       tiles number between half and 6 times the device's resident warps (FP32 grids
                        of about 2K to 12K per side), else kernel 2 (tdepth 4) whenever it can.  All
-                       kernels round every operation the same way, so the FP32 states do not
-                       depend on the choice */
-  int32_t rows;     /* rows per CTA (kernels 1, 3) or per warp tile (kernels 2, 4); 0 = auto */
+                       kernels round every operation the same way, so the states do not depend on
+                       the choice */
+  int32_t rows;     /* rows per CTA (kernels 1, 3) or per warp tile (kernels 2, 4, FP64); 0 = auto */
   int32_t tdepth;   /* steps per pass of kernels 2 and 3 (0 = default); leftover steps run one per pass */
   int32_t reserved; /* 0.  Bits 0 and 1 are test hooks of the failure detection: with bit 0
                        kernel 3 never issues one row copy, with bit 1 kernel 4 never reports

@@ -38,8 +38,8 @@ class TsunamiFn(torch.autograd.Function):
                 raise ValueError(f"{name} must have shape (ny, ld) = {(g.ny, g.ld)} (got {tuple(t.shape)})")
         med = tsu.Medium(tsu._field(hx, g, code, "hx"), tsu._field(hy, g, code, "hy"), float(cfg.ext[1]),
                          float(cfg.ext[3]), float(cfg.ext[0]), float(cfg.ext[2]))
-        # four state buffers: FP32 runs then take the warp-blocked pass (receivers and checkpoints
-        # recorded by it), FP64 runs one step per pass
+        # four state buffers: FP32 runs then take the on-chip pass where the grid fits, or else the
+        # warp-blocked pass (receivers and checkpoints recorded by it)
         bufs = [torch.zeros_like(u0) for _ in range(4)]
         st = tsu.State()
         for k, b in enumerate(bufs):
