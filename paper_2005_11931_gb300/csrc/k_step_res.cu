@@ -17,7 +17,7 @@
 // windows, as k_step_wtb.cu does, takes 100 to 176), and one exchange, about 2 us, per four steps.
 // Measured (GB300, us per step, before and after): 769^2 with receivers 4.1 and 1.35; 1024^2 3.6 and
 // 1.43, 1400^2 4.6 and 1.9, 2048^2 5.9 and 4.7; with the energy 1003 x 517 4.8 and 1.7, 1024^2 4.9 and
-// 2.0, 1536^2 5.7 and 3.0, 2048^2 6.85 and 6.05.
+// 1.8, 1536^2 5.7 and 3.0, 2048^2 6.85 and 6.05.
 //
 // All warps run the row code in step (a barrier per step): when only neighbouring warps waited for
 // each other they drifted apart, and the unrolled code of all of them no longer fitted the
@@ -96,15 +96,21 @@ constexpr int kTmemRows = 16;
 // barrier more per step, between the chains and the next rows), the rims' staging shares their
 // place, and the chains' results of a pass wait in the workspace.
 constexpr bool res_lean(int R, bool ENERGY) { return ENERGY && R > 12; }
+// Tiles of up to 8 rows per warp keep the terms of all the steps of a pass and add them up at its end,
+// four chains at a time, while the rims travel, instead of one step behind the rows: 1024^2 1.82 against
+// 1.93 us per step, 1200^2 2.30 against 2.50; at 10 rows 3.18 against 3.02.
+constexpr bool res_batch(int R, bool ENERGY) { return ENERGY && R <= 8; }
 template <int R, bool WIDE, bool ENERGY>
 struct ResSmem {
-  static constexpr bool kLean = res_lean(R, ENERGY);
+  static constexpr bool kLean = res_lean(R, ENERGY), kBatch = res_batch(R, ENERGY);
   static constexpr int kStage = 4 * R > 32 ? 4 * R : 32;
   float4 xch[2][kResWarps][2][32];   // first and last u row of every warp, double buffered
-  // energy: the terms of the last two steps summed over each lane's columns, the (sum, error) of each
+  // energy: the terms of the last steps summed over each lane's columns, the (sum, error) of each
   // thread's chain of rows for the pass's steps, and those of each warp
-  alignas(16) float er[ENERGY && !kLean ? 2 : 1][ENERGY ? kResWarps * R : 1][32];
-  float2 es[ENERGY && !kLean ? kResK : 1][ENERGY && !kLean ? kResThreads : 1];
+  static constexpr int kEr = kBatch ? kResK : ENERGY && !kLean ? 2 : 1;
+  static constexpr bool kEs = ENERGY && !kLean && !kBatch;
+  alignas(16) float er[kEr][ENERGY ? kResWarps * R : 1][32];
+  float2 es[kEs ? kResK : 1][kEs ? kResThreads : 1];
   float2 esw[kResK][kResWarps];
   int2 rec[kResMaxRec];              // (row << 8 | column in the tile, receiver)
   // per warp: one row of u, or the values of its first and last output lanes on their way
@@ -201,7 +207,7 @@ __device__ __forceinline__ void pair_add(float2& a, const float2 b) {
 template <int R, int RB, bool WIDE, bool ENERGY, bool REC>
 __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a) {
   using Smem = ResSmem<R, WIDE, ENERGY>;
-  constexpr bool LEAN = Smem::kLean;
+  constexpr bool LEAN = Smem::kLean, BATCH = Smem::kBatch;
   static_assert(!LEAN || !REC, "no place to stage receivers");
   static_assert(!LEAN || sizeof(Smem::er) >= sizeof(float4) * kResWarps * Smem::kStage, "staging");
   extern __shared__ __align__(16) unsigned char res_raw[];
@@ -341,7 +347,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
     if (col_out) {
 #pragma unroll 4
       for (int r = r0; r < r1; ++r) {
-        const float y = sm.er[LEAN ? 0 : s & 1][r][lane] - ec;
+        const float y = sm.er[s % Smem::kEr][r][lane] - ec;
         const float sum = es + y;
         ec = (sum - es) - y;
         es = sum;
@@ -349,7 +355,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
     }
     if constexpr (LEAN)
       a.es[((int64_t)cta * kResK + s) * kResThreads + tid] = make_float2(es, -ec);
-    else
+    else if constexpr (Smem::kEs)
       sm.es[s][tid] = make_float2(es, -ec);
   };
 
@@ -369,7 +375,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       const P4 below = w > 0 ? as_p4(sm.xch[buf][w - 1][1][lane]) : zero;
       const P4 above = w + 1 < kResWarps ? as_p4(sm.xch[buf][w + 1][0][lane]) : zero;
       buf ^= 1;
-      if constexpr (ENERGY) {
+      if constexpr (ENERGY && !BATCH) {
         if (s > 0) {
           chain(s - 1);
           if constexpr (LEAN) __syncthreads();
@@ -471,7 +477,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
               u[r].p[q] = add2(u[r].p[q], vn.p[q]);
             }
             set_v(r, vn);
-            if constexpr (ENERGY) sm.er[LEAN ? 0 : s & 1][w * R + r][lane] = erow;
+            if constexpr (ENERGY) sm.er[s % Smem::kEr][w * R + r][lane] = erow;
           }
           gb = gy[RB - 1];
         }
@@ -532,16 +538,37 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       }
     }
     if constexpr (ENERGY) {
-      if constexpr (!LEAN) {
+      float2 e[kResK];
+      if constexpr (BATCH) {
+        __syncthreads();
+        float es[kResK], ec[kResK];
+#pragma unroll
+        for (int t = 0; t < kResK; ++t) es[t] = ec[t] = 0.f;
+        const int r0 = kResK + kResChain * w, r1 = min(r0 + kResChain, kResK + y1 - y0);
+        if (col_out) {
+#pragma unroll 2
+          for (int r = r0; r < r1; ++r)
+#pragma unroll
+            for (int t = 0; t < kResK; ++t) {  // steps past ns hold older terms, dropped below
+              const float y = sm.er[t % Smem::kEr][r][lx] - ec[t];
+              const float sum = es[t] + y;
+              ec[t] = (sum - es[t]) - y;
+              es[t] = sum;
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < kResK; ++t) e[t] = t < ns ? make_float2(es[t], -ec[t]) : make_float2(0.f, 0.f);
+      } else if constexpr (!LEAN) {
         __syncthreads();
         chain(ns - 1);
       }
       // the warp's sums of the pass's steps: lanes 8 t .. 8 t + 7 end up with step t
-      float2 e[kResK];
+      if constexpr (!BATCH) {
 #pragma unroll
-      for (int t = 0; t < kResK; ++t) {
-        e[t] = make_float2(0.f, 0.f);
-        if (t < ns) e[t] = LEAN ? a.es[((int64_t)cta * kResK + t) * kResThreads + tx] : sm.es[LEAN ? 0 : t][LEAN ? 0 : tx];
+        for (int t = 0; t < kResK; ++t) {
+          e[t] = make_float2(0.f, 0.f);
+          if (t < ns) e[t] = LEAN ? a.es[((int64_t)cta * kResK + t) * kResThreads + tx] : sm.es[Smem::kEs ? t : 0][Smem::kEs ? tx : 0];
+        }
       }
       auto fold = [&](float2& keep, const float2& send, int o) {
         pair_add(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, o), __shfl_xor_sync(0xffffffffu, send.y, o)));
@@ -661,7 +688,8 @@ const ResVariant kResVariants[] = {
     res_variant<8, 2, true, false>(),  res_variant<10, 2, true, false>(), res_variant<12, 2, true, false>(),
     res_variant<14, 2, true, false>(),  res_variant<17, 2, true, false>(), res_variant<2, 2, false, true>(),
     res_variant<3, 3, false, true>(),   res_variant<4, 2, false, true>(),  res_variant<5, 2, true, true>(),
-    res_variant<6, 2, true, true>(),   res_variant<8, 2, true, true>(),  res_variant<10, 2, true, true>(),
+    res_variant<6, 2, true, true>(),   res_variant<7, 2, true, true>(),  res_variant<8, 2, true, true>(),
+    res_variant<10, 2, true, true>(),
     res_variant<12, 2, true, true>(),   res_variant<14, 2, true, true>(),  res_variant<17, 2, true, true>()};
 constexpr int kResPlain = 11;  // variants without the energy
 constexpr int kResNumVariants = (int)(sizeof kResVariants / sizeof kResVariants[0]);

@@ -44,7 +44,8 @@ def run(nx, ny, calls, kernel, energy=False, nrec=0, spoil=None):
 # without the energy (12 with it); the last ones are too large for either
 SIZES = [(2001, ny) for ny in (130, 249, 300, 381, 400, 500, 561, 630, 700, 800, 881, 900, 1100, 1139, 1350, 1401,
                                1600, 2000, 2046)]
-SIZES += [(64, 64), (65, 34), (97, 3001), (120, 130), (121, 2449), (3001, 97), (1025, 1023), (2200, 1700)]
+SIZES += [(3, 3), (4, 70), (5, 200), (64, 64), (65, 34), (97, 3001), (120, 130), (121, 2449), (3001, 97), (1025, 1023), (2200, 1700)]
+SIZES += [(64, 723), (130, 724), (64, 725)]  # a last chunk of 1, 2, 3 rows: halos reach past it
 
 
 @pytest.mark.parametrize("nx,ny", SIZES)
