@@ -136,3 +136,40 @@ def test_checkpoints(dtype, nx, ny, every, calls):
         out.append((sim.u.clone(), other.clone(), ck, tr))
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+def test_several_streams_and_threads():
+    """Resident launches of several problems from several threads and streams at once: each waits only
+    for its own CTAs, so they give what they give one after another."""
+    import threading
+
+    cases = [("f32", 1025, 900), ("f32", 300, 200), ("f64", 201, 201), ("f64", 500, 499)]
+
+    def build(dtype, nx, ny):
+        sim = tsu.Simulation.create(nx, DEPTH, dtype=dtype, ny=ny)
+        u0 = tsu.empty_field(sim.g, dtype)
+        u0[1:-1, 1 : nx - 1] = torch.from_numpy(np.random.default_rng(nx).standard_normal((ny - 2, nx - 2))).to(u0.dtype)
+        sim.init(u0)
+        return sim
+
+    alone, together = [build(*c) for c in cases], [build(*c) for c in cases]
+    torch.cuda.synchronize()
+    for sim in alone:
+        for _ in range(5):
+            sim.step(200)
+    torch.cuda.synchronize()
+
+    def work(sim):
+        s = torch.cuda.Stream()
+        for _ in range(5):
+            sim.step(200, stream=s)
+        s.synchronize()
+
+    threads = [threading.Thread(target=work, args=(sim,)) for sim in together]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for a, b in zip(alone, together):
+        tsu.tsu_sync_status(b.ws, b.ws.numel())
+        assert torch.equal(a.u, b.u)
