@@ -28,8 +28,8 @@ struct A64Args {
   const double* u;  // u^n of the first step; u^{n-k} at u - k ustride
   int64_t ustride;
   int rows, nstrips, nchunks, nsteps;
-  uint4* col;
-  uint4* row;
+  ulonglong2* col;
+  ulonglong2* row;
   const int64_t* rec_idx;
   int32_t nrec;
   const double* g;  // g^n of the first step; g^{n-k} at g - k nrec
@@ -174,13 +174,13 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_adjoint_res64(const A64Args 
     __syncthreads();
     if (cnt > 0) {
       const bool edge = (lane == 0 && has_l) || (lane == 31 && has_r);
-      const uint4* cs = col_rim(q, lane == 0 ? cta - 1 : cta + 1, lane == 0 ? 1 : 0);
-      uint4 x[R], xd, xu;
+      const ulonglong2* cs = col_rim(q, lane == 0 ? cta - 1 : cta + 1, lane == 0 ? 1 : 0);
+      ulonglong2 x[R], xd, xu;
 #pragma unroll
       for (int r = 0; r < R; ++r)
         if (edge && r < cnt) x[r] = try64(cs + r);
       const bool dn = w == 0 && has_d && node, up = w == wl && has_u && node;
-      const uint4 *ds = row_rim(q, cta - nsx, 1), *us = row_rim(q, cta + nsx, 0);
+      const ulonglong2 *ds = row_rim(q, cta - nsx, 1), *us = row_rim(q, cta + nsx, 0);
       if (dn) xd = try64(ds);
       if (up) xu = try64(us);
       if (w > 0) below = sm.xch[q][w - 1][1][lane];
@@ -271,7 +271,7 @@ cudaError_t launch_adjoint_res64(const StencilGeom& g, const void* hx, const voi
   a.nstrips = (int)strips;
   a.nchunks = (int)((inner + rows - 1) / rows);
   a.nsteps = (int)nsteps;
-  a.col = (uint4*)ws;
+  a.col = (ulonglong2*)ws;
   a.row = a.col + (int64_t)2 * a.nstrips * a.nchunks * 2 * kR64Rows;
   a.rec_idx = rec_idx;
   a.nrec = nrec;

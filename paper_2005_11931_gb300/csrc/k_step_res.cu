@@ -61,9 +61,11 @@ constexpr uint64_t kResWaitNs = 10000000000ull;
 
 // One lane's four columns of u and v as they travel between CTAs: every 8 bytes hold a value and
 // the number of the pass that wrote it, so a reader polls the data itself and no flag, fence or
-// barrier stands between the store and its use (8-byte accesses are single-copy atomic).
+// barrier stands between the store and its use.  The accesses are vectors of two 64-bit elements: an
+// aligned 8-byte element is read and written whole, while of a vector of 32-bit elements the memory
+// model would allow a reader to see the tag without the value.
 struct alignas(16) ResItem {
-  uint32_t w[16];
+  uint64_t w[8];  // value | tag << 32
 };
 static_assert(sizeof(ResItem) == 64, "item");
 
@@ -130,10 +132,12 @@ __device__ __forceinline__ float4 as_f4(const P4& v) {
 __device__ __forceinline__ float4 ldcg4(const float* g, bool ok) {
   return ok ? __ldcg(reinterpret_cast<const float4*>(g)) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
+__device__ __forceinline__ uint64_t tagged(float x, const uint32_t tag) {
+  return (uint64_t)tag << 32 | __float_as_uint(x);
+}
 __device__ __forceinline__ void item_put(ResItem* d, const float4& u, const float4& v, const uint32_t tag) {
   auto st = [&](int k, float x, float y) {
-    asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %2};" ::"l"(&d->w[4 * k]), "r"(__float_as_uint(x)),
-                 "r"(tag), "r"(__float_as_uint(y))
+    asm volatile("st.volatile.global.v2.b64 [%0], {%1, %2};" ::"l"(&d->w[2 * k]), "l"(tagged(x, tag)), "l"(tagged(y, tag))
                  : "memory");
   };
   st(0, u.x, u.y);
@@ -142,18 +146,19 @@ __device__ __forceinline__ void item_put(ResItem* d, const float4& u, const floa
   st(3, v.z, v.w);
 }
 __device__ __forceinline__ bool item_try(const ResItem* d, float4& u, float4& v, const uint32_t tag) {
-  uint32_t x[16];
+  uint64_t x[8];
 #pragma unroll
   for (int k = 0; k < 4; ++k)
-    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(x[4 * k]), "=r"(x[4 * k + 1]), "=r"(x[4 * k + 2]), "=r"(x[4 * k + 3])
-                 : "l"(&d->w[4 * k])
+    asm volatile("ld.volatile.global.v2.b64 {%0, %1}, [%2];"
+                 : "=l"(x[2 * k]), "=l"(x[2 * k + 1])
+                 : "l"(&d->w[2 * k])
                  : "memory");
-  u = make_float4(__uint_as_float(x[0]), __uint_as_float(x[2]), __uint_as_float(x[4]), __uint_as_float(x[6]));
-  v = make_float4(__uint_as_float(x[8]), __uint_as_float(x[10]), __uint_as_float(x[12]), __uint_as_float(x[14]));
+  auto value = [&](int k) { return __uint_as_float((uint32_t)x[k]); };
+  u = make_float4(value(0), value(1), value(2), value(3));
+  v = make_float4(value(4), value(5), value(6), value(7));
   bool ok = true;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) ok = ok && x[2 * k + 1] == tag;
+  for (int k = 0; k < 8; ++k) ok = ok && (uint32_t)(x[k] >> 32) == tag;
   return ok;
 }
 // bounded wait for an item of pass `tag` (its CTA is resident: cooperative launch); dead: a wait

@@ -43,8 +43,8 @@ struct R64Args {
   int rows, nstrips, nchunks;
   int64_t nsteps;
   double* part;  // [step][CTA] energy partials
-  uint4* col;    // [2][CTA][2][kR64Rows] first and last own column
-  uint4* row;    // [2][CTA][2][32] first and last own row
+  ulonglong2* col;    // [2][CTA][2][kR64Rows] first and last own column
+  ulonglong2* row;    // [2][CTA][2][32] first and last own row
   int* status;
   double* traces;
   int32_t nrec;
@@ -188,13 +188,13 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_leapfrog_res64(const R64Args
       if (cnt > 0) {
         // the neighbours' edges: every load issued before the first is waited for
         const bool edge = (lane == 0 && has_l) || (lane == 31 && has_r);
-        const uint4* cs = col_rim(q, lane == 0 ? cta - 1 : cta + 1, lane == 0 ? 1 : 0);
-        uint4 x[R], xd, xu;
+        const ulonglong2* cs = col_rim(q, lane == 0 ? cta - 1 : cta + 1, lane == 0 ? 1 : 0);
+        ulonglong2 x[R], xd, xu;
 #pragma unroll
         for (int r = 0; r < R; ++r)
           if (edge && r < cnt) x[r] = try64(cs + r);
         const bool dn = w == 0 && has_d && node, up = w == wl && has_u && node;
-        const uint4 *ds = row_rim(q, cta - nsx, 1), *us = row_rim(q, cta + nsx, 0);
+        const ulonglong2 *ds = row_rim(q, cta - nsx, 1), *us = row_rim(q, cta + nsx, 0);
         if (dn) xd = try64(ds);
         if (up) xu = try64(us);
         if (w > 0) below = sm.xch[q][w - 1][1][lane];
@@ -319,7 +319,7 @@ static R64Args r64_args(const StencilGeom& g, const void* hx, const void* hy, co
   a.rows = (int)rows;
   a.nstrips = (int)r64_strips(g.nx);
   a.nchunks = (int)((g.ny - 2 + rows - 1) / rows);
-  a.col = (uint4*)rims;
+  a.col = (ulonglong2*)rims;
   a.row = a.col + (int64_t)2 * a.nstrips * a.nchunks * 2 * kR64Rows;
   return a;
 }

@@ -12,37 +12,37 @@ constexpr int kR64Out = 30;    // own columns of a strip: 30 s + 1 .. 30 s + 30
 constexpr int kR64Rows = 128;  // most rows of a tile
 constexpr uint64_t kR64WaitNs = 10000000000ull;
 // rims: [2][CTA][2][kR64Rows] first and last own column, [2][CTA][2][32] first and last own row
-constexpr size_t kR64RimBytes = (size_t)2 * kResMaxCtas * 2 * (kR64Rows + 32) * sizeof(uint4);
+constexpr size_t kR64RimBytes = (size_t)2 * kResMaxCtas * 2 * (kR64Rows + 32) * sizeof(ulonglong2);
 inline int64_t r64_strips(int64_t nx) { return (nx - 2 + kR64Out - 1) / kR64Out; }
 
-__device__ __forceinline__ void put64(uint4* d, const double x, const uint32_t tag) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %2};" ::"l"(d), "r"((uint32_t)b), "r"(tag),
-               "r"((uint32_t)(b >> 32))
-               : "memory");
+// A double travels as two 64-bit words, each half of it with the tag in the upper 32 bits (an aligned 8-byte
+// element of a vector access is read and written whole, a 32-bit one would be on its own).
+__device__ __forceinline__ void put64(ulonglong2* d, const double x, const uint32_t tag) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x), t = (unsigned long long)tag << 32;
+  asm volatile("st.volatile.global.v2.b64 [%0], {%1, %2};" ::"l"(d), "l"(t | (uint32_t)b), "l"(t | b >> 32) : "memory");
 }
-__device__ __forceinline__ uint4 try64(const uint4* d) {
-  uint4 x;
-  asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w)
-               : "l"(d)
-               : "memory");
+__device__ __forceinline__ ulonglong2 try64(const ulonglong2* d) {
+  ulonglong2 x;
+  asm volatile("ld.volatile.global.v2.b64 {%0, %1}, [%2];" : "=l"(x.x), "=l"(x.y) : "l"(d) : "memory");
   return x;
 }
+__device__ __forceinline__ bool has_tag(const ulonglong2& x, const uint32_t tag) {
+  return (uint32_t)(x.x >> 32) == tag && (uint32_t)(x.y >> 32) == tag;
+}
 // the value of x, read again until both its halves carry the tag (bounded)
-__device__ __forceinline__ double get64(uint4 x, const uint4* d, const uint32_t tag, bool& dead) {
-  if (!(x.y == tag && x.w == tag) && !dead) {
+__device__ __forceinline__ double get64(ulonglong2 x, const ulonglong2* d, const uint32_t tag, bool& dead) {
+  if (!has_tag(x, tag) && !dead) {
     const uint64_t t0 = global_ns();
     long long it = 0;
     for (; it < kSpinCap; ++it) {
       x = try64(d);
-      if (x.y == tag && x.w == tag) break;
+      if (has_tag(x, tag)) break;
       if ((it & 63) == 63 && global_ns() - t0 > kR64WaitNs) it = kSpinCap;
     }
     dead = it >= kSpinCap;
   }
   if (dead) return __longlong_as_double(0x7ff8000000000000ll);  // a wait ran out: nothing that follows is valid
-  return __longlong_as_double((long long)((unsigned long long)x.z << 32 | x.x));
+  return __longlong_as_double((long long)(x.y << 32 | (uint32_t)x.x));
 }
 
 }  // namespace dev
