@@ -33,6 +33,8 @@ struct A64Args {
   const int64_t* rec_idx;
   int32_t nrec;
   const double* g;  // g^n of the first step; g^{n-k} at g - k nrec
+  PollLimit wait;
+  uint32_t skew;  // added to the tags sent: 0 (test hook: a number that no reader waits for)
 };
 
 struct A64Smem {
@@ -160,14 +162,14 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_adjoint_res64(const A64Args 
 #pragma unroll
     for (int r = 0; r < R; ++r)
       if (r < cnt && ((lane == 1 && has_l) || (lane == 30 && has_r)))
-        put64(col_rim(q, cta, lane == 30 ? 1 : 0) + r, l[r], tag);
+        put64(col_rim(q, cta, lane == 30 ? 1 : 0) + r, l[r], tag + a.skew);
     double top = l[0];
 #pragma unroll
     for (int r = 1; r < R; ++r)
       if (r < cnt) top = l[r];
     if (cnt > 0) {
-      if (w == 0 && has_d) put64(row_rim(q, cta, 0), l[0], tag);
-      if (w == wl && has_u) put64(row_rim(q, cta, 1), top, tag);
+      if (w == 0 && has_d) put64(row_rim(q, cta, 0), l[0], tag + a.skew);
+      if (w == wl && has_u) put64(row_rim(q, cta, 1), top, tag + a.skew);
       sm.xch[q][w][0][lane] = l[0];
       sm.xch[q][w][1][lane] = top;
     }
@@ -187,9 +189,9 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_adjoint_res64(const A64Args 
       if (w < wl) above = sm.xch[q][w + 1][0][lane];
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        if (edge && r < cnt) l[r] = get64(x[r], cs + r, tag, dead);
-      if (dn) below = get64(xd, ds, tag, dead);
-      if (up) above = get64(xu, us, tag, dead);
+        if (edge && r < cnt) l[r] = get64(x[r], cs + r, tag, a.wait, dead);
+      if (dn) below = get64(xd, ds, tag, a.wait, dead);
+      if (up) above = get64(xu, us, tag, a.wait, dead);
       __syncwarp();
     }
   }
@@ -243,7 +245,7 @@ int a64_sms() {
 cudaError_t launch_adjoint_res64(const StencilGeom& g, const void* hx, const void* hy, void* lam, void* lam_pp,
                                  const void* u, int64_t ustride, void* gx, void* gy, int32_t nrec,
                                  const int64_t* rec_idx, const void* gv, int64_t nsteps, void* ws, cudaStream_t s,
-                                 bool* ran) {
+                                 bool hold, bool* ran) {
   *ran = false;
   const int64_t sms = a64_sms(), strips = r64_strips(g.nx), inner = g.ny - 2;
   if (!ws || sms <= 0 || strips < 1 || strips > sms || g.ny >= 1 << 22 || nsteps < 2 || nsteps > 16384 ||
@@ -276,6 +278,8 @@ cudaError_t launch_adjoint_res64(const StencilGeom& g, const void* hx, const voi
   a.rec_idx = rec_idx;
   a.nrec = nrec;
   a.g = (const double*)gv;
+  a.wait = r64_limit(ws, hold);
+  a.skew = hold ? 1u << 31 : 0u;
   // no value may carry a tag of an earlier launch
   cudaError_t e = cudaMemsetAsync(ws, 0, kR64RimBytes, s);
   if (e != cudaSuccess) return e;

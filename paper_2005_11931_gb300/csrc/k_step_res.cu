@@ -57,7 +57,6 @@ constexpr int kResChain = 16;  // rows of an energy chain (k_step_wtb.cu's small
 // A launch never runs longer than a fraction of a second, so that another resident launch on the
 // device, whose CTAs may be placed as this one's leave, gets its SMs well inside the bound of its waits.
 constexpr int64_t kResMaxSteps = 16384;
-constexpr uint64_t kResWaitNs = 10000000000ull;
 
 // One lane's four columns of u and v as they travel between CTAs: every 8 bytes hold a value and
 // the number of the pass that wrote it, so a reader polls the data itself and no flag, fence or
@@ -90,6 +89,8 @@ struct ResArgs {
   int32_t nrec;
   const int* rec_off;
   const int4* rec_ent;
+  PollLimit wait;
+  uint32_t skew;  // added to the tags sent: 0 (test hook: a number that no reader waits for)
 };
 
 // rows r < kTmemRows of a wide tile keep their faces in tensor memory
@@ -163,12 +164,13 @@ __device__ __forceinline__ bool item_try(const ResItem* d, float4& u, float4& v,
 }
 // bounded wait for an item of pass `tag` (its CTA is resident: cooperative launch); dead: a wait
 // ran out before, take what is there
-__device__ __forceinline__ void item_get(const ResItem* d, float4& u, float4& v, const uint32_t tag, bool& dead) {
+__device__ __forceinline__ void item_get(const ResItem* d, float4& u, float4& v, const uint32_t tag, const PollLimit& w,
+                                         bool& dead) {
   if (item_try(d, u, v, tag) || dead) return;
   const uint64_t t0 = global_ns();
-  for (long long it = 0; it < kSpinCap; ++it) {
+  for (int it = 0; it < kPollCap; ++it) {
     if (item_try(d, u, v, tag)) return;
-    if ((it & 63) == 63 && global_ns() - t0 > kResWaitNs) break;
+    if (poll_over(w, it, t0)) break;
   }
   dead = true;
 }
@@ -533,8 +535,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
         for (int r = 0; r < R; ++r) {
           if (!((rim_rows >> r) & 1u)) continue;
           const int j = rx + r;
-          if (j < y0 + kResK) item_put(row_rim(q, cta, 0, j - y0) + lx, as_f4(u[r]), as_f4(get_v(r)), tag);
-          if (j >= y1 - kResK) item_put(row_rim(q, cta, 1, j - (y1 - kResK)) + lx, as_f4(u[r]), as_f4(get_v(r)), tag);
+          if (j < y0 + kResK) item_put(row_rim(q, cta, 0, j - y0) + lx, as_f4(u[r]), as_f4(get_v(r)), tag + a.skew);
+          if (j >= y1 - kResK) item_put(row_rim(q, cta, 1, j - (y1 - kResK)) + lx, as_f4(u[r]), as_f4(get_v(r)), tag + a.skew);
         }
       }
       __syncwarp();
@@ -548,7 +550,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       __syncwarp();
       for (int k = lx; k < 2 * R; k += 32)
         if ((k & 1) ? has_r : has_l)
-          item_put(col_rim(q, cta, k & 1) + (k >> 1), stage[2 * k], stage[2 * k + 1], tag);
+          item_put(col_rim(q, cta, k & 1) + (k >> 1), stage[2 * k], stage[2 * k + 1], tag + a.skew);
     } else if (col_out) {  // ---- the end: the whole tile
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -645,7 +647,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       }
       if (src) {
         float4 x, y;
-        item_get(src, x, y, tag, dead);
+        item_get(src, x, y, tag, a.wait, dead);
         dst[0] = x;
         dst[1] = y;
       }
@@ -753,8 +755,9 @@ int64_t res_strips(int64_t ld) { return (ld + 4 + kResOut - 1) / kResOut; }
 
 // Workspace of the resident pass for this grid: counters, rims and partials of the largest of the
 // variants whose tiles number at most kResMaxCtas; 0: the grid does not fit on any device.
+// the rims, then 128 bytes with the word of expired waits (PollLimit)
 static size_t res_rim_bytes(int k, int64_t ncta) {
-  return (size_t)ncta * 2 * (2 * kResWarps * kResVariants[k].rows + 2 * kResK * 32) * sizeof(ResItem);
+  return (size_t)ncta * 2 * (2 * kResWarps * kResVariants[k].rows + 2 * kResK * 32) * sizeof(ResItem) + 128;
 }
 static size_t res_part_bytes(int k, int64_t ncta) {
   const bool lean = res_lean(kResVariants[k].rows, k >= kResPlain);
@@ -796,7 +799,7 @@ bool res_fits(const StencilGeom& g, bool energy) {
 
 cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
                             double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
-                            const int64_t* rec_idx, void* traces, bool table, bool* ran, int* last) {
+                            const int64_t* rec_idx, void* traces, bool table, bool hold, bool* ran, int* last) {
   *ran = false;
   *last = 0;
   int k = 0;
@@ -827,6 +830,8 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
   a.part = (double*)((char*)ews.res + res_rim_bytes(k, ncta));
   a.es = (float2*)(a.part + kResEnergySteps * ncta);
   a.status = ews.status;
+  a.wait = PollLimit{hold ? kPollHookNs : kPollNs, (int*)((char*)ews.res + res_rim_bytes(k, ncta) - 128)};
+  a.skew = hold ? 1u << 31 : 0u;
   cudaError_t e = cudaSuccess;
   if (traces && nrec > 0) {
     if (table) e = launch_wtb_rec_table(g, rows, rec_idx, nrec, ews, s);

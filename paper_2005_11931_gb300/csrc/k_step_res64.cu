@@ -51,6 +51,8 @@ struct R64Args {
   const int64_t* rec_idx;
   double* seg;  // or nullptr: u^{n+1+k} into seg + k seg_stride, and u, p left as they are
   int64_t seg_stride;
+  PollLimit wait;
+  uint32_t skew;  // added to the tags sent: 0 (test hook: a number that no reader waits for)
 };
 
 struct R64Smem {
@@ -173,14 +175,14 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_leapfrog_res64(const R64Args
 #pragma unroll
       for (int r = 0; r < R; ++r)
         if (r < cnt && ((lane == 1 && has_l) || (lane == 30 && has_r)))
-          put64(col_rim(q, cta, lane == 30 ? 1 : 0) + r, u[r], tag);
+          put64(col_rim(q, cta, lane == 30 ? 1 : 0) + r, u[r], tag + a.skew);
       double top = u[0];
 #pragma unroll
       for (int r = 1; r < R; ++r)
         if (r < cnt) top = u[r];
       if (cnt > 0) {
-        if (w == 0 && has_d) put64(row_rim(q, cta, 0), u[0], tag);
-        if (w == wl && has_u) put64(row_rim(q, cta, 1), top, tag);
+        if (w == 0 && has_d) put64(row_rim(q, cta, 0), u[0], tag + a.skew);
+        if (w == wl && has_u) put64(row_rim(q, cta, 1), top, tag + a.skew);
         sm.xch[q][w][0][lane] = u[0];
         sm.xch[q][w][1][lane] = top;
       }
@@ -201,9 +203,9 @@ __global__ void __launch_bounds__(kR64Threads, 1) k_leapfrog_res64(const R64Args
         if (w < wl) above = sm.xch[q][w + 1][0][lane];
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          if (edge && r < cnt) u[r] = get64(x[r], cs + r, tag, dead);
-        if (dn) below = get64(xd, ds, tag, dead);
-        if (up) above = get64(xu, us, tag, dead);
+          if (edge && r < cnt) u[r] = get64(x[r], cs + r, tag, a.wait, dead);
+        if (dn) below = get64(xd, ds, tag, a.wait, dead);
+        if (up) above = get64(xu, us, tag, a.wait, dead);
         __syncwarp();
       }
     }
@@ -305,8 +307,10 @@ bool res64_fits(const StencilGeom& g, const EnergyWs& ews) {
 }
 
 static R64Args r64_args(const StencilGeom& g, const void* hx, const void* hy, const void* u, const void* p, int64_t rows,
-                        void* rims) {
+                        void* rims, bool hold) {
   R64Args a{};
+  a.wait = r64_limit(rims, hold);
+  a.skew = hold ? 1u << 31 : 0u;
   a.nx = g.nx;
   a.ny = g.ny;
   a.ld = g.ld;
@@ -343,12 +347,12 @@ static cudaError_t r64_launch(const R64Args& a, R64Kernel kern, cudaStream_t s) 
 
 cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* hy, void* u, void* p, double* energy,
                               const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
-                              const int64_t* rec_idx, void* traces, bool* ran) {
+                              const int64_t* rec_idx, void* traces, bool hold, bool* ran) {
   *ran = false;
   int64_t rows = 0;
   const int k = r64_workspace(ews) ? r64_plan(g, &rows) : -1;
   if (k < 0 || nsteps >= 1ll << 31 || (traces && nrec > kResMaxRec)) return cudaSuccess;
-  R64Args a = r64_args(g, hx, hy, u, p, rows, ews.res);
+  R64Args a = r64_args(g, hx, hy, u, p, rows, ews.res, hold);
   a.part = (double*)((char*)ews.res + kR64RimBytes);
   a.status = ews.status;
   a.nrec = traces ? nrec : 0;
@@ -372,12 +376,13 @@ size_t res64_seg_bytes(const StencilGeom& g) {
 }
 
 cudaError_t launch_step_res64_seg(const StencilGeom& g, const void* hx, const void* hy, const void* u, const void* p,
-                                  void* seg, int64_t seg_stride, int64_t nsteps, void* ws, cudaStream_t s, bool* ran) {
+                                  void* seg, int64_t seg_stride, int64_t nsteps, void* ws, cudaStream_t s, bool hold,
+                                  bool* ran) {
   *ran = false;
   int64_t rows = 0;
   const int k = ws ? r64_plan(g, &rows) : -1;
   if (k < 0 || nsteps < 1 || nsteps > kR64MaxSteps) return cudaSuccess;
-  R64Args a = r64_args(g, hx, hy, u, p, rows, ws);
+  R64Args a = r64_args(g, hx, hy, u, p, rows, ws, hold);
   a.nsteps = nsteps;
   a.seg = (double*)seg;
   a.seg_stride = seg_stride;

@@ -10,9 +10,12 @@ namespace dev {
 constexpr int kR64Warps = 8, kR64Threads = kR64Warps * 32;
 constexpr int kR64Out = 30;    // own columns of a strip: 30 s + 1 .. 30 s + 30
 constexpr int kR64Rows = 128;  // most rows of a tile
-constexpr uint64_t kR64WaitNs = 10000000000ull;
-// rims: [2][CTA][2][kR64Rows] first and last own column, [2][CTA][2][32] first and last own row
-constexpr size_t kR64RimBytes = (size_t)2 * kResMaxCtas * 2 * (kR64Rows + 32) * sizeof(ulonglong2);
+// rims: [2][CTA][2][kR64Rows] first and last own column, [2][CTA][2][32] first and last own row; the word of
+// expired waits (PollLimit) in the last 128 bytes
+constexpr size_t kR64RimBytes = (size_t)2 * kResMaxCtas * 2 * (kR64Rows + 32) * sizeof(ulonglong2) + 128;
+inline PollLimit r64_limit(void* rims, bool hold) {
+  return PollLimit{hold ? kPollHookNs : kPollNs, (int*)((char*)rims + kR64RimBytes - 128)};
+}
 inline int64_t r64_strips(int64_t nx) { return (nx - 2 + kR64Out - 1) / kR64Out; }
 
 // A double travels as two 64-bit words, each half of it with the tag in the upper 32 bits (an aligned 8-byte
@@ -30,16 +33,19 @@ __device__ __forceinline__ bool has_tag(const ulonglong2& x, const uint32_t tag)
   return (uint32_t)(x.x >> 32) == tag && (uint32_t)(x.y >> 32) == tag;
 }
 // the value of x, read again until both its halves carry the tag (bounded)
-__device__ __forceinline__ double get64(ulonglong2 x, const ulonglong2* d, const uint32_t tag, bool& dead) {
+__device__ __forceinline__ double get64(ulonglong2 x, const ulonglong2* d, const uint32_t tag, const PollLimit& w,
+                                        bool& dead) {
   if (!has_tag(x, tag) && !dead) {
     const uint64_t t0 = global_ns();
-    long long it = 0;
-    for (; it < kSpinCap; ++it) {
+    dead = true;
+    for (int it = 0; it < kPollCap; ++it) {
       x = try64(d);
-      if (has_tag(x, tag)) break;
-      if ((it & 63) == 63 && global_ns() - t0 > kR64WaitNs) it = kSpinCap;
+      if (has_tag(x, tag)) {
+        dead = false;
+        break;
+      }
+      if (poll_over(w, it, t0)) break;
     }
-    dead = it >= kSpinCap;
   }
   if (dead) return __longlong_as_double(0x7ff8000000000000ll);  // a wait ran out: nothing that follows is valid
   return __longlong_as_double((long long)(x.y << 32 | (uint32_t)x.x));

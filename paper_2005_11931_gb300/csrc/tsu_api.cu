@@ -395,6 +395,7 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   const bool res64 = dtype == TSU_F64 && st->form == TSU_FORM_STANDARD && have_ws;
   if (o.kernel == 0 && o.rows == 0 && (res32 || res64) && (!o.traces || o.nrec <= tsu::kResMaxRec)) {
     const int64_t nres = res32 && o.energy ? nsteps / 4 * 4 : nsteps;
+    const bool hold = (o.reserved & 4) != 0;
     bool ran = true;
     while (ran && k < nres) {
       const int64_t due = o.ckpt ? ((st->step - 1) % o.ckpt_every + o.ckpt_every) % o.ckpt_every : 0;  // 0: now
@@ -410,9 +411,10 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
         e = checkpoint(st, o, field_bytes, s);
       int last = 0;
       if (e == cudaSuccess)
-        e = res32 ? tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, en, ews, n, s, o.nrec, o.rec_idx, tr, k == 0, &ran,
-                                         &last)
-                  : tsu::launch_step_res64(sg, m->hx, m->hy, uu[0], vv[0], en, ews, n, s, o.nrec, o.rec_idx, tr, &ran);
+        e = res32 ? tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, en, ews, n, s, o.nrec, o.rec_idx, tr, k == 0, hold,
+                                         &ran, &last)
+                  : tsu::launch_step_res64(sg, m->hx, m->hy, uu[0], vv[0], en, ews, n, s, o.nrec, o.rec_idx, tr, hold,
+                                           &ran);
       if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n resident launch");
       if (!ran) break;
       if (last == 1) {
@@ -651,10 +653,12 @@ int64_t tsu_ckpt_slots(int64_t nsteps, int64_t ckpt_every) {
   return (nsteps - 2) / ckpt_every + 1;
 }
 
-int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_medium* m, int64_t nsteps,
-                int64_t ckpt_every, const void* ckpt, const void* u0, int32_t nrec, const int64_t* rec_idx,
-                const void* dtraces, double* g_hx, double* g_hy, void* g_u0, void* g_u1, void* ws, size_t ws_bytes,
-                void* stream) {
+// tsu_adjoint with test hooks of the failure detection, for the tests only (not in tsu.h): with bit 2 of
+// `hooks` no CTA of the FP64 recompute on chip recognises its neighbours' edges, with bit 3 none of the sweep.
+int tsu_adjoint_hooks(const tsu_grid* g, int dtype, int form, double tau, const tsu_medium* m, int64_t nsteps,
+                      int64_t ckpt_every, const void* ckpt, const void* u0, int32_t nrec, const int64_t* rec_idx,
+                      const void* dtraces, double* g_hx, double* g_hy, void* g_u0, void* g_u1, void* ws,
+                      size_t ws_bytes, int32_t hooks, void* stream) {
   g_err[0] = 0;
   TRY(check_grid(g));
   TRY(check_dtype(dtype));
@@ -801,7 +805,7 @@ int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_me
     if (dtype == TSU_F64 && form == TSU_FORM_STANDARD && mend - mc >= kResMinSteps) {
       bool ran = false;  // the whole segment in one launch where the grid fits on chip
       e = tsu::launch_step_res64_seg(sg, m->hx, m->hy, segp(b, 0), extra(b), segp(b, 1), (int64_t)(fb / es), mend - mc,
-                                     res_ws, aux->s, &ran);
+                                     res_ws, aux->s, (hooks & 4) != 0, &ran);
       if (e != cudaSuccess) return cuda_fail(e, "tsu_adjoint recompute");
       if (ran) k = mend - mc;
     }
@@ -824,7 +828,7 @@ int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_me
       bool ran = false;
       e = tsu::launch_adjoint_res64(sg, m->hx, m->hy, lam4[i1], lam4[i2], segp(b, mend - mc), (int64_t)(fb / es), accx,
                                     accy, nrec, rec_idx, nrec > 0 ? (const char*)dtraces + (size_t)(mend - 1) * nrec * es : nullptr,
-                                    mend - nlo + 1, res_ws ? res_ws + res_b : nullptr, s, &ran);
+                                    mend - nlo + 1, res_ws ? res_ws + res_b : nullptr, s, (hooks & 8) != 0, &ran);
       if (e != cudaSuccess) return cuda_fail(e, "tsu_adjoint resident sweep");
       if (ran) n_first = nlo - 1;
     }
@@ -858,6 +862,14 @@ int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_me
   if (e == cudaSuccess && dtype == TSU_F32) e = tsu::launch_flush(sg, accx, accy, g_hx, g_hy, s);
   if (e != cudaSuccess) return cuda_fail(e, "tsu_adjoint start");
   return TSU_OK;
+}
+
+int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_medium* m, int64_t nsteps,
+                int64_t ckpt_every, const void* ckpt, const void* u0, int32_t nrec, const int64_t* rec_idx,
+                const void* dtraces, double* g_hx, double* g_hy, void* g_u0, void* g_u1, void* ws, size_t ws_bytes,
+                void* stream) {
+  return tsu_adjoint_hooks(g, dtype, form, tau, m, nsteps, ckpt_every, ckpt, u0, nrec, rec_idx, dtraces, g_hx, g_hy,
+                           g_u0, g_u1, ws, ws_bytes, 0, stream);
 }
 
 // ---------------------------------------------------------------------------------------------

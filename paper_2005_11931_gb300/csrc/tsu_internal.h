@@ -63,11 +63,13 @@ constexpr int32_t kResMaxRec = 512;  // receivers a CTA keeps in its list
 size_t res_bytes(int64_t ny, int64_t ld);  // 0: the grid does not fit
 // nsteps steps (FP32, increment form): from (u, v)[0], using (u, v)[1] as the other pair;
 // the state ends up in (u, v)[*last].  table: build the receiver table (the first launch of a call).
-//   energy and traces per step, or nullptr.  *ran = false and
-// nothing enqueued when the device, the workspace or the grid do not allow it.
+// energy and traces per step, or nullptr.  hold: the failure-detection test hook (tsu_step_opts.reserved
+// bit 2) of this and the following launches: no CTA recognises what its neighbours send, and its waits
+// expire after 20 ms.
+// *ran = false and nothing enqueued when the device, the workspace or the grid do not allow it.
 cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
                             double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
-                            const int64_t* rec_idx, void* traces, bool table, bool* ran, int* last);
+                            const int64_t* rec_idx, void* traces, bool table, bool hold, bool* ran, int* last);
 bool res_fits(const StencilGeom& g, bool energy);  // on this device
 
 // The same for FP64 grids of up to about 750^2 in the standard form (k_step_res64.cu): u = u^n and
@@ -75,19 +77,20 @@ bool res_fits(const StencilGeom& g, bool energy);  // on this device
 size_t res64_bytes(int64_t ny, int64_t ld);
 cudaError_t launch_step_res64(const StencilGeom& g, const void* hx, const void* hy, void* u, void* p, double* energy,
                               const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
-                              const int64_t* rec_idx, void* traces, bool* ran);
+                              const int64_t* rec_idx, void* traces, bool hold, bool* ran);
 bool res64_fits(const StencilGeom& g, const EnergyWs& ews);
 // the same storing every state, u^{n+1+k} into seg + k seg_stride (elements), u = u^n and p = u^{n-1} left
 // as they are; ws: res64_seg_bytes(g) bytes (0: the grid does not fit).  A wait that ran out leaves NaN.
 size_t res64_seg_bytes(const StencilGeom& g);
 cudaError_t launch_step_res64_seg(const StencilGeom& g, const void* hx, const void* hy, const void* u, const void* p,
-                                  void* seg, int64_t seg_stride, int64_t nsteps, void* ws, cudaStream_t s, bool* ran);
+                                  void* seg, int64_t seg_stride, int64_t nsteps, void* ws, cudaStream_t s, bool hold,
+                                  bool* ran);
 // nsteps reverse steps (k_adjoint_res64.cu) from lam = lam^{n+1}, lam_pp = lam^{n+2} (in place) with u^{n-k} at
 // u - k ustride and the receivers' values of step k at gv - k nrec; ws: res64_seg_bytes(g) bytes of its own
 cudaError_t launch_adjoint_res64(const StencilGeom& g, const void* hx, const void* hy, void* lam, void* lam_pp,
                                  const void* u, int64_t ustride, void* gx, void* gy, int32_t nrec,
                                  const int64_t* rec_idx, const void* gv, int64_t nsteps, void* ws, cudaStream_t s,
-                                 bool* ran);
+                                 bool hold, bool* ran);
 
 // receivers the warp-blocked pass records itself (longer lists go one step per pass)
 constexpr int32_t kWtbMaxReceivers = 2048;
