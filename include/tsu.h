@@ -267,6 +267,8 @@ int tsu_adjoint_workspace(const tsu_grid* g, int dtype, int form, int64_t nsteps
  * host thread, created by that thread's first call and destroyed when the thread exits)
  * concurrently with the reverse sweep of the previous one; all of it is ordered before the
  * call's last work on the caller's stream.
+ * FP64 grids that fit on chip take bounded waits here too (as tsu_step_n's automatic choice).  There is no
+ * status word: one that runs out leaves NaN in the gradients that depend on it.
  * Errors: TSU_EINVAL, TSU_ENONPOS, TSU_ECFL, TSU_ENOMEM, TSU_ECUDA. */
 int tsu_adjoint(const tsu_grid* g, int dtype, int form, double tau, const tsu_medium* m, int64_t nsteps,
                 int64_t ckpt_every, const void* ckpt, const void* u0, int32_t nrec, const int64_t* rec_idx,
@@ -339,7 +341,8 @@ const char* tsu_noalloc_last_error(void);
 
 /* Synchronise the stream, then read and clear the device status word in the workspace of
  * tsu_step_n or of the implicit calls: TSU_OK, or TSU_ETIMEOUT if a bounded device-side wait of a
- * kernel expired (that kernel stopped early; its outputs are invalid). */
+ * kernel expired.  The outputs of that call are invalid: the kernel stopped early or, in the passes on
+ * chip, went on with NaN in the place of what did not arrive. */
 int tsu_sync_status(void* ws, size_t ws_bytes, void* stream);
 
 /* Energy E^{n-1/2} of the current pair (u^{n-1}, u^n) into energy_dev[0] (device double, or NULL)

@@ -162,17 +162,21 @@ __device__ __forceinline__ bool item_try(const ResItem* d, float4& u, float4& v,
   for (int k = 0; k < 8; ++k) ok = ok && (uint32_t)(x[k] >> 32) == tag;
   return ok;
 }
-// bounded wait for an item of pass `tag` (its CTA is resident: cooperative launch); dead: a wait
-// ran out before, take what is there
+// The item of pass `tag`, waited for with a bound (its CTA is resident: cooperative launch).  dead: a wait ran
+// out, now or before; what is not there is NaN, so that no result of it looks valid.
 __device__ __forceinline__ void item_get(const ResItem* d, float4& u, float4& v, const uint32_t tag, const PollLimit& w,
                                          bool& dead) {
-  if (item_try(d, u, v, tag) || dead) return;
-  const uint64_t t0 = global_ns();
-  for (int it = 0; it < kPollCap; ++it) {
-    if (item_try(d, u, v, tag)) return;
-    if (poll_over(w, it, t0)) break;
+  if (item_try(d, u, v, tag)) return;
+  if (!dead) {
+    const uint64_t t0 = global_ns();
+    for (int it = 0; it < kPollCap; ++it) {
+      if (item_try(d, u, v, tag)) return;
+      if (poll_over(w, it, t0)) break;
+    }
   }
   dead = true;
+  const float nan = __uint_as_float(0x7fffffffu);
+  u = v = make_float4(nan, nan, nan, nan);
 }
 // ---- tensor memory as a scratchpad: 8 columns of the warp's 32 lanes per call -------------------
 struct Tm8 {

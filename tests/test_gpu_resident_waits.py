@@ -58,6 +58,21 @@ def test_forward(dtype, nx, ny, energy):
         assert torch.equal(x, y)
 
 
+# a call of two passes and one of several: what is not NaN does not depend on what never arrived
+@pytest.mark.parametrize("nx,ny", [(300, 200), (1200, 1100), (1500, 1500), (2001, 2000)])
+@pytest.mark.parametrize("energy", [False, True])
+@pytest.mark.parametrize("steps", [8, 24])
+def test_forward_leaves_no_valid_looking_values(nx, ny, energy, steps):
+    sim, u0 = problem("f32", nx, ny)
+    u, v = expired(sim, u0, steps, energy)
+    assert u.isnan().any() and v.isnan().any()
+    sim.init(u0)
+    sim.step(steps, kernel=1)
+    for x, y in ((u, sim.u), (v, sim.v)):
+        ok = ~x.isnan()
+        assert torch.equal(x[ok], y[ok])
+
+
 def adjoint(sim, u0, S, every, hooks):
     """Gradients of a seeded receiver functional; hooks: see tsu_adjoint_hooks."""
     g = sim.g
