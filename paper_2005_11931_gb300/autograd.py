@@ -5,6 +5,7 @@ steps through libtsu, recording ``u^n`` at the receivers for n = 1..S (a [S, nre
 checkpointing the state every ``cfg.ckpt_every`` steps.  ``backward`` hands dJ/dtraces to
 ``tsu_adjoint``, which recomputes each checkpoint segment and runs the reverse-time adjoint, and
 returns dJ/dhx, dJ/dhy (FP64 accumulated, cast to the field type), dJ/du0 and dJ/du1.
+``sync_status(traces)`` reports a bounded wait of the forward run that ran out.
 Marshalling only: all arithmetic is in the CUDA kernels.
 """
 from __future__ import annotations
@@ -25,6 +26,7 @@ class TsunamiConfig:
     ext: tuple                 # face extrema [min hx, max hx, min hy, max hy] (from tsu_make_depth)
     form: int = tsu.TSU_FORM_INCREMENT
     ckpt_every: int = 64
+    debug: int = 0             # tsu_step_opts.reserved of the forward run (test hooks)
 
 
 class TsunamiFn(torch.autograd.Function):
@@ -56,10 +58,12 @@ class TsunamiFn(torch.autograd.Function):
             o = tsu.StepOpts()
             o.nrec, o.rec_idx, o.traces = nrec, cfg.rec_idx.data_ptr(), traces.data_ptr()
             o.ckpt, o.ckpt_every, o.ckpt_slots = ckpt.data_ptr(), int(cfg.ckpt_every), slots
+            o.reserved = int(cfg.debug)
             tsu.tsu_step_n(g, code, cfg.tau, med, st, S - 1, o, ws, ws_b)
         tsu.tsu_observe(g, code, cfg.tau, med, st, None, cfg.rec_idx, traces[S - 1], ws, ws_b)
         ctx.save_for_backward(hx, hy, u0, ckpt)
         ctx.cfg = cfg
+        ctx.status_ws = ws  # holds the status word of the run's bounded waits: sync_status
         return traces
 
     @staticmethod
@@ -90,3 +94,13 @@ def tsunami_traces(hx, hy, u0, u1, cfg: TsunamiConfig) -> torch.Tensor:
     if u1 is None:
         u1 = torch.zeros_like(u0)
     return TsunamiFn.apply(hx, hy, u0, u1, cfg)
+
+
+def sync_status(traces: torch.Tensor, stream=None):
+    """Synchronise and raise TsuError (TSU_ETIMEOUT) if a bounded device-side wait of the forward run that
+    recorded ``traces`` (as returned by tsunami_traces, with a gradient) ran out.  Nothing synchronises
+    otherwise: such a run leaves NaN in the fields, and in the traces and gradients that depend on them."""
+    fn = traces.grad_fn
+    if not hasattr(fn, "status_ws"):
+        raise ValueError("traces must be the tensor tsunami_traces returned for inputs that require a gradient")
+    tsu.tsu_sync_status(fn.status_ws, fn.status_ws.numel(), stream)

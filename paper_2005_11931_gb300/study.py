@@ -109,6 +109,7 @@ def reflected_pulse(eps: float, n: int = 769, T: float = 0.45, amp: float = 1.0,
         s.step(steps - 1, rec_idx=rec, traces=tr[: steps - 1])
         s.observe(rec_idx=rec, trace=tr[steps - 1])
         traces.append(tr[:, 0].double().cpu().numpy())
+        tsu.tsu_sync_status(s.ws, s.ws.numel())
     t = sim.tau * np.arange(1, steps + 1)
     scattered = traces[0] - traces[1]
     inc = int(np.argmax(np.abs(traces[1])))
@@ -157,5 +158,7 @@ def misfit_eps_gradient(n: int, depth: dict, u0: np.ndarray, S: int, rec_ij: np.
     out = torch.zeros(1, dtype=torch.float64, device="cuda")
     rws = torch.empty(tsu.tsu_reduce_workspace(), dtype=torch.uint8, device="cuda")
     tsu.tsu_depth_eps_gradient(g, depth, gx, gy, out, rws)
+    for s in (obs_sim, sim):
+        tsu.tsu_sync_status(s.ws, s.ws.numel())
     return {"J": 0.5 * float((res.double() ** 2).sum()), "dJ_deps": float(out), "tau": sim.tau,
             "observed": obs.double().cpu().numpy()}
