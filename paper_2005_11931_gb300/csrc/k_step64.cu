@@ -39,31 +39,15 @@ __device__ __forceinline__ double b64(const S64Geom& g, double fr, double fl, do
 }
 
 // FORM 0: standard (p = u^{n-1}, out = u^{n+1}, may be written over p); FORM 1: increment (p = v^n updated
-// in place, out = u^{n+1})
-template <int FORM, bool STORE, bool ENERGY>
+// in place, out = u^{n+1}).  MANY: several tiles per warp, where the caller has no room for one energy
+// partial per four tiles (the loop costs 0.5 % at 2048^2, so the other launches do without).
+template <int FORM, bool STORE, bool ENERGY, bool MANY = false>
 __global__ void __launch_bounds__(kS64Warps * 32) k_leapfrog64(const S64Geom g, const double* __restrict__ hx,
                                                                const double* __restrict__ hy,
                                                                const double* u, const double* p_in,
                                                                double* p_out, double* u_next, const PassOut o,
                                                                const double escale) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int tile = blockIdx.x * kS64Warps + w;
-  const int chunk = tile / g.strips, strip = tile - chunk * g.strips;
-  const int c = strip * kS64Out + lane - 1;
-  const int j0 = 1 + chunk * g.rows, j1 = tile < g.ntiles ? min(j0 + g.rows, g.ny - 1) : j0;
-  const bool in = c >= 0 && c < g.nx;
-  double fx[kS64Batch], fy[kS64Batch], hd = 0.0;
-  auto faces = [&](int jb) {
-#pragma unroll
-    for (int k = 0; k < kS64Batch; ++k) {
-      const int64_t q = (int64_t)(jb + k) * g.ld + c;
-      const bool ok = in && jb + k < j1;
-      fx[k] = ok ? __ldg(hx + q) : 0.0;
-      fy[k] = ok ? __ldg(hy + q) : 0.0;
-    }
-  };
-  faces(j0);
-  if (in && j0 < j1) hd = __ldg(hy + (int64_t)(j0 - 1) * g.ld + c);
   // receivers: u^n at the receiver nodes, by the first CTA (u is read-only in this pass)
   if (o.trace && blockIdx.x == 0) {
     const int64_t total = (int64_t)g.ny * g.ld;
@@ -73,7 +57,23 @@ __global__ void __launch_bounds__(kS64Warps * 32) k_leapfrog64(const S64Geom g, 
     }
   }
   double es = 0.0, ec = 0.0;  // compensated energy sum of this lane
-  if (j0 < j1) {
+  for (int tile = blockIdx.x * kS64Warps + w; tile < g.ntiles; tile += gridDim.x * kS64Warps) {
+    const int chunk = tile / g.strips, strip = tile - chunk * g.strips;
+    const int c = strip * kS64Out + lane - 1;
+    const int j0 = 1 + chunk * g.rows, j1 = min(j0 + g.rows, g.ny - 1);
+    const bool in = c >= 0 && c < g.nx;
+    double fx[kS64Batch], fy[kS64Batch], hd = 0.0;
+    auto faces = [&](int jb) {
+#pragma unroll
+      for (int k = 0; k < kS64Batch; ++k) {
+        const int64_t q = (int64_t)(jb + k) * g.ld + c;
+        const bool ok = in && jb + k < j1;
+        fx[k] = ok ? __ldg(hx + q) : 0.0;
+        fy[k] = ok ? __ldg(hy + q) : 0.0;
+      }
+    };
+    faces(j0);
+    if (in) hd = __ldg(hy + (int64_t)(j0 - 1) * g.ld + c);
     const bool out = lane >= 1 && c <= g.nx - 2;  // the strips cover columns 0 .. nx - 2
     const bool node = out && c >= 1;
     const bool tail = lane == 31 && c + 1 < g.nx;
@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kS64Warps * 32) k_leapfrog64(const S64Geom g, 
         }
       }
     }
+    if constexpr (!MANY) break;
   }
   if constexpr (ENERGY) {
     __shared__ double red[kS64Warps];
@@ -305,14 +306,18 @@ template <int FORM>
 cudaError_t step64(const StencilGeom& g, const void* hx, const void* hy, const void* p, const void* u, void* v,
                    void* u_next, const PassOut& o, bool store, int rows, cudaStream_t s) {
   const S64Geom q = s64_geom(g, rows);
-  const unsigned grid = (unsigned)((q.ntiles + kS64Warps - 1) / kS64Warps);
+  int64_t grid = (q.ntiles + kS64Warps - 1) / kS64Warps;
   const double scale = g.dxdy / (2.0 * g.tau * g.tau);
-  if (o.energy && !o.defer && grid > o.ews.capacity) return cudaErrorInvalidValue;
+  const bool many = o.energy && !o.defer && grid > o.ews.capacity;
+  if (many) grid = o.ews.capacity;
+  if (grid < 1) return cudaErrorInvalidValue;
   auto run = [&](auto kern) {
-    kern<<<grid, kS64Warps * 32, 0, s>>>(q, (const double*)hx, (const double*)hy, (const double*)u, (const double*)p,
-                                         (double*)v, (double*)u_next, o, scale);
+    kern<<<(unsigned)grid, kS64Warps * 32, 0, s>>>(q, (const double*)hx, (const double*)hy, (const double*)u,
+                                                   (const double*)p, (double*)v, (double*)u_next, o, scale);
   };
-  if (o.energy)
+  if (many)
+    store ? run(k_leapfrog64<FORM, true, true, true>) : run(k_leapfrog64<FORM, false, true, true>);
+  else if (o.energy)
     store ? run(k_leapfrog64<FORM, true, true>) : run(k_leapfrog64<FORM, false, true>);
   else
     store ? run(k_leapfrog64<FORM, true, false>) : run(k_leapfrog64<FORM, false, false>);

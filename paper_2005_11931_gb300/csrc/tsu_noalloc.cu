@@ -27,7 +27,8 @@ namespace {
 
 // At most this many CTAs of the one-step pass (one FP64 partial each): with 128 threads x one
 // 16-byte vector per thread and 32 rows per CTA this covers every grid with
-// ceil(ld / 512) * ceil((ny - 2) / 32) <= 65536 in FP32 (e.g. 16384^2) and half of that in FP64.
+// ceil(ld / 512) * ceil((ny - 2) / 32) <= 65536 in FP32 (e.g. 16384^2) and half of that in FP64 (whose
+// tiles are narrower: where they are more than the array holds, a CTA takes several).
 constexpr int64_t kNoallocPartials = 65536;
 constexpr size_t kNoallocBytes = 256 + (size_t)kNoallocPartials * sizeof(double);  // 512 KiB + 256 B
 constexpr int kNoallocRows = 32;
@@ -110,9 +111,6 @@ int tsu_step_n_noalloc(const tsu_grid* g, int dtype, double tau, const tsu_mediu
   sg.cy = tau * tau / (g->dy * g->dy);
   sg.tau = tau;
   sg.dxdy = g->dx * g->dy;
-  // FP64 tiles are narrower than the count above assumes: more rows each where that is too many
-  int rows = kNoallocRows;
-  while (dtype == TSU_F64 && tsu::step64_ctas(g->nx, g->ny, rows) > kNoallocPartials) rows *= 2;
   for (int64_t k = 0; k < nsteps; ++k) {
     tsu::PassOut po{};
     po.energy = energy ? energy + k : nullptr;
@@ -120,13 +118,13 @@ int tsu_step_n_noalloc(const tsu_grid* g, int dtype, double tau, const tsu_mediu
     cudaError_t e;
     if (st->form == TSU_FORM_STANDARD) {
       e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, st->buf[st->aux], st->buf[st->cur], nullptr,
-                           st->buf[st->aux], po, true, rows, s);
+                           st->buf[st->aux], po, true, kNoallocRows, s);
     } else {
       int f = -1;
       for (int b = 0; b < st->nbuf && f < 0; ++b)
         if (b != st->cur && b != st->aux) f = b;
       e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, nullptr, st->buf[st->cur], st->buf[st->aux],
-                           st->buf[f], po, true, rows, s);
+                           st->buf[f], po, true, kNoallocRows, s);
       if (e == cudaSuccess) st->cur = f;
     }
     if (e != cudaSuccess) return na_fail(TSU_ECUDA, cudaGetErrorString(e));
