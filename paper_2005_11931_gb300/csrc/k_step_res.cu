@@ -796,9 +796,22 @@ static int res_rows(int64_t ny, int64_t ld, bool energy, int* variant) {
   return 0;
 }
 
-bool res_fits(const StencilGeom& g, bool energy) {
-  int k = 0;
-  return res_rows(g.ny, g.ld, energy, &k) > 0;
+// The variant and the rows per CTA for these outputs (rec: receivers are recorded); false: the device, the
+// workspace or the grid do not allow it.
+static bool res_plan(const StencilGeom& g, bool energy, bool rec, int32_t nrec, const EnergyWs& ews, int* variant,
+                     int* rows) {
+  if (energy) {  // the rows that the pass taken otherwise sums its energy over
+    const bool flow = !rec && wtb_flow_preferred(g.ny, g.ld);
+    if ((flow ? wtb_flow_rows(g.ny, g.ld) : wtb_auto_rows(g.ny, g.ld, kResK)) != kResChain) return false;
+  }
+  *rows = res_rows(g.ny, g.ld, energy, variant);
+  return *rows > 0 && ews.res && ews.res_size >= res_bytes(g.ny, g.ld) && ews.status && (!rec || nrec <= kResMaxRec) &&
+         kResVariants[*variant].kern[rec ? 1 : 0];
+}
+
+bool res_fits(const StencilGeom& g, bool energy, bool rec, int32_t nrec, const EnergyWs& ews) {
+  int k = 0, rows = 0;
+  return res_plan(g, energy, rec, nrec, ews, &k, &rows);
 }
 
 cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
@@ -806,14 +819,9 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
                             const int64_t* rec_idx, void* traces, bool table, bool hold, bool* ran, int* last) {
   *ran = false;
   *last = 0;
-  int k = 0;
-  if (energy) {  // the rows that the pass taken otherwise sums its energy over
-    const bool flow = !traces && wtb_flow_preferred(g.ny, g.ld);
-    if ((flow ? wtb_flow_rows(g.ny, g.ld) : wtb_auto_rows(g.ny, g.ld, kResK)) != kResChain) return cudaSuccess;
-  }
-  const int rows = res_rows(g.ny, g.ld, energy != nullptr, &k);
-  if (rows == 0 || !ews.res || ews.res_size < res_bytes(g.ny, g.ld) || !ews.status || nsteps < 1 || nsteps >= (int64_t)1 << 31 ||
-      (traces && nrec > kResMaxRec))
+  int k = 0, rows = 0;
+  if (nsteps < 1 || nsteps >= (int64_t)1 << 31 ||
+      !res_plan(g, energy != nullptr, traces != nullptr, nrec, ews, &k, &rows))
     return cudaSuccess;
   ResArgs a{};
   a.nx = g.nx;
@@ -827,7 +835,6 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
   a.nstrips = (int)res_strips(g.ld);
   a.nchunks = (g.ny - 2 + rows - 1) / rows;
   const ResVariant& x = kResVariants[k];
-  if (!x.kern[traces && nrec > 0 ? 1 : 0]) return cudaSuccess;
   const int64_t ncta = (int64_t)a.nstrips * a.nchunks;
   a.col = (ResItem*)ews.res;
   a.row = a.col + 2 * ncta * 2 * kResWarps * x.rows;
@@ -837,7 +844,7 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
   a.wait = PollLimit{hold ? kPollHookNs : kPollNs, (int*)((char*)ews.res + res_rim_bytes(k, ncta) - 128)};
   a.skew = hold ? 1u << 31 : 0u;
   cudaError_t e = cudaSuccess;
-  if (traces && nrec > 0) {
+  if (traces) {
     if (table) e = launch_wtb_rec_table(g, rows, rec_idx, nrec, ews, s);
     if (e == cudaSuccess) e = launch_wtb_trace_edges(g, rec_idx, nrec, traces, nsteps, s);
     if (e != cudaSuccess) return e;

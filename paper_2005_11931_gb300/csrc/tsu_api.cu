@@ -388,35 +388,91 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   const size_t field_bytes = (size_t)g->ny * g->ld * elem_size(dtype);
   cudaStream_t s = (cudaStream_t)stream;
   int64_t k = 0;
+  // FP64 steps with the energy: the CTAs' partials of several steps are kept (in the region the FP32
+  // resident pass has) and summed by one launch, instead of by the last CTA of every step, which on
+  // small grids costs as much as the step
+  const int64_t ctas64 = dtype == TSU_F64 ? tsu::step64_ctas(g->nx, g->ny, o.rows) : 0;
+  const int64_t keep = ctas64 > 0 && ctas64 <= 1024 && o.energy && ews.res
+                           ? std::min<int64_t>(256, (int64_t)(ews.res_size / (ctas64 * sizeof(double))))
+                           : 0;
+  auto one_step_passes = [&](int64_t end) -> int {  // steps k .. end - 1, one per launch
+    int64_t kept = 0;
+    for (; k < end; ++k) {
+      tsu::PassOut po{};
+      po.energy = o.energy ? o.energy + k : nullptr;
+      po.ews = ews;
+      if (keep > 1) po.defer = (double*)ews.res + kept * ctas64;
+      po.nrec = o.nrec;
+      po.rec_idx = o.rec_idx;
+      po.trace = o.traces ? (char*)o.traces + (size_t)k * o.nrec * elem_size(dtype) : nullptr;
+      const int64_t n = st->step;  // state holds u^n
+      if (o.ckpt && ((n - 1) % o.ckpt_every) == 0 && (n - 1) / o.ckpt_every < o.ckpt_slots) {
+        char* slot = (char*)o.ckpt + (size_t)((n - 1) / o.ckpt_every) * 2 * field_bytes;
+        po.ckpt_a = slot;
+        po.ckpt_b = slot + field_bytes;
+      }
+      cudaError_t e;
+      if (st->form == TSU_FORM_STANDARD) {
+        e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, st->buf[st->aux], st->buf[st->cur], nullptr,
+                             st->buf[st->aux], po, true, (use_tb || use_wtb) ? 0 : o.rows, s);
+      } else {
+        const int f = scratch_index(st, -1);
+        e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, nullptr, st->buf[st->cur], st->buf[st->aux],
+                             st->buf[f], po, true, (use_tb || use_wtb) ? 0 : o.rows, s);
+      }
+      if (e == cudaSuccess && po.defer && (++kept == keep || k + 1 == end)) {
+        e = tsu::launch_energy64(sg, (const double*)ews.res, ctas64, kept, o.energy + (k + 1 - kept), s);
+        kept = 0;
+      }
+      if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n launch");
+      if (st->form == TSU_FORM_STANDARD) {
+        const int t = st->cur;
+        st->cur = st->aux;
+        st->aux = t;
+      } else {
+        st->cur = scratch_index(st, -1);
+      }
+      st->step += 1;
+    }
+    return TSU_OK;
+  };
   // Grids whose fields fit on chip: every step up to the next checkpoint in one cooperative launch.  FP32
   // with the energy: the last nsteps % 4 steps go one per pass as after the blocked passes (the one-step
   // pass rounds the energy's terms differently), and with checkpoints too the blocked passes run.
   const bool res32 = flow_base && !(o.energy && o.ckpt);
   const bool res64 = dtype == TSU_F64 && st->form == TSU_FORM_STANDARD && have_ws;
-  if (o.kernel == 0 && o.rows == 0 && (res32 || res64) && (!o.traces || o.nrec <= tsu::kResMaxRec)) {
+  const bool fits = o.kernel == 0 && o.rows == 0 && (res32 || res64) && (!o.traces || o.nrec <= tsu::kResMaxRec) &&
+                    (res32 ? tsu::res_fits(sg, o.energy != nullptr, o.traces != nullptr, o.nrec, ews)
+                           : tsu::res64_fits(sg, ews));
+  if (fits) {
     const int64_t nres = res32 && o.energy ? nsteps / 4 * 4 : nsteps;
     const bool hold = (o.reserved & 4) != 0;
-    bool ran = true;
+    bool ran = true, table = true;
     while (ran && k < nres) {
       const int64_t due = o.ckpt ? ((st->step - 1) % o.ckpt_every + o.ckpt_every) % o.ckpt_every : 0;  // 0: now
       const int64_t n = o.ckpt && o.ckpt_every - due < nres - k ? o.ckpt_every - due : nres - k;
-      if (n < kResMinSteps) break;
+      if (n < kResMinSteps) {
+        // a short stretch up to a checkpoint does not keep those after it from running on chip
+        if (nres - k - n < kResMinSteps || o.ckpt_every < kResMinSteps) break;
+        TRY(one_step_passes(k + n));
+        continue;
+      }
       const int f1 = scratch_index(st, -1), f2 = scratch_index(st, f1);
       void* const uu[2] = {st->buf[st->cur], res32 ? st->buf[f1] : nullptr};
       void* const vv[2] = {st->buf[st->aux], res32 ? st->buf[f2] : nullptr};
       void* tr = o.traces ? (char*)o.traces + (size_t)k * o.nrec * elem_size(dtype) : nullptr;
       double* en = o.energy ? o.energy + k : nullptr;
       cudaError_t e = cudaSuccess;
-      if (o.ckpt && due == 0 && (res32 ? tsu::res_fits(sg, o.energy != nullptr) : tsu::res64_fits(sg, ews)))
-        e = checkpoint(st, o, field_bytes, s);
+      if (o.ckpt && due == 0) e = checkpoint(st, o, field_bytes, s);
       int last = 0;
       if (e == cudaSuccess)
-        e = res32 ? tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, en, ews, n, s, o.nrec, o.rec_idx, tr, k == 0, hold,
+        e = res32 ? tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, en, ews, n, s, o.nrec, o.rec_idx, tr, table, hold,
                                          &ran, &last)
                   : tsu::launch_step_res64(sg, m->hx, m->hy, uu[0], vv[0], en, ews, n, s, o.nrec, o.rec_idx, tr, hold,
                                            &ran);
       if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n resident launch");
       if (!ran) break;
+      table = false;
       if (last == 1) {
         st->cur = f1;
         st->aux = f2;
@@ -484,52 +540,7 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
       st->step += tdepth;
     }
   }
-  // FP64 steps with the energy: the CTAs' partials of several steps are kept (in the region the FP32
-  // resident pass has) and summed by one launch, instead of by the last CTA of every step, which on
-  // small grids costs as much as the step
-  const int64_t ctas64 = dtype == TSU_F64 ? tsu::step64_ctas(g->nx, g->ny, o.rows) : 0;
-  const int64_t keep = ctas64 > 0 && ctas64 <= 1024 && o.energy && ews.res
-                           ? std::min<int64_t>(256, (int64_t)(ews.res_size / (ctas64 * sizeof(double))))
-                           : 0;
-  int64_t kept = 0;
-  for (; k < nsteps; ++k) {
-    tsu::PassOut po{};
-    po.energy = o.energy ? o.energy + k : nullptr;
-    po.ews = ews;
-    if (keep > 1) po.defer = (double*)ews.res + kept * ctas64;
-    po.nrec = o.nrec;
-    po.rec_idx = o.rec_idx;
-    po.trace = o.traces ? (char*)o.traces + (size_t)k * o.nrec * elem_size(dtype) : nullptr;
-    const int64_t n = st->step;  // state holds u^n
-    if (o.ckpt && ((n - 1) % o.ckpt_every) == 0 && (n - 1) / o.ckpt_every < o.ckpt_slots) {
-      char* slot = (char*)o.ckpt + (size_t)((n - 1) / o.ckpt_every) * 2 * field_bytes;
-      po.ckpt_a = slot;
-      po.ckpt_b = slot + field_bytes;
-    }
-    cudaError_t e;
-    if (st->form == TSU_FORM_STANDARD) {
-      e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, st->buf[st->aux], st->buf[st->cur], nullptr,
-                           st->buf[st->aux], po, true, (use_tb || use_wtb) ? 0 : o.rows, s);
-    } else {
-      const int f = scratch_index(st, -1);
-      e = tsu::launch_step(sg, dtype, st->form, m->hx, m->hy, nullptr, st->buf[st->cur], st->buf[st->aux],
-                           st->buf[f], po, true, (use_tb || use_wtb) ? 0 : o.rows, s);
-    }
-    if (e == cudaSuccess && po.defer && (++kept == keep || k + 1 == nsteps)) {
-      e = tsu::launch_energy64(sg, (const double*)ews.res, ctas64, kept, o.energy + (k + 1 - kept), s);
-      kept = 0;
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "tsu_step_n launch");
-    if (st->form == TSU_FORM_STANDARD) {
-      const int t = st->cur;
-      st->cur = st->aux;
-      st->aux = t;
-    } else {
-      st->cur = scratch_index(st, -1);
-    }
-    st->step += 1;
-  }
-  return TSU_OK;
+  return one_step_passes(nsteps);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -70,7 +70,8 @@ size_t res_bytes(int64_t ny, int64_t ld);  // 0: the grid does not fit
 cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
                             double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
                             const int64_t* rec_idx, void* traces, bool table, bool hold, bool* ran, int* last);
-bool res_fits(const StencilGeom& g, bool energy);  // on this device
+// whether such a call runs on chip on this device (rec: with traces)
+bool res_fits(const StencilGeom& g, bool energy, bool rec, int32_t nrec, const EnergyWs& ews);
 
 // The same for FP64 grids of up to about 750^2 in the standard form (k_step_res64.cu): u = u^n and
 // p = u^{n-1} are updated in place.
