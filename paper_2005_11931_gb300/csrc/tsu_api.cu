@@ -449,8 +449,15 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
     const bool hold = (o.reserved & 4) != 0;
     bool ran = true, table = true;
     while (ran && k < nres) {
-      const int64_t due = o.ckpt ? ((st->step - 1) % o.ckpt_every + o.ckpt_every) % o.ckpt_every : 0;  // 0: now
-      const int64_t n = o.ckpt && o.ckpt_every - due < nres - k ? o.ckpt_every - due : nres - k;
+      // n steps up to the next checkpoint; now: one is due before them.  A full store takes none.
+      int64_t n = nres - k;
+      bool now = false;
+      if (o.ckpt) {
+        const int64_t past = ((st->step - 1) % o.ckpt_every + o.ckpt_every) % o.ckpt_every;
+        const int64_t slot = (st->step - 1 - past) / o.ckpt_every;  // of the last one at or before this step
+        now = past == 0 && slot < o.ckpt_slots;
+        if (slot + 1 < o.ckpt_slots && o.ckpt_every - past < n) n = o.ckpt_every - past;
+      }
       if (n < kResMinSteps) {
         // a short stretch up to a checkpoint does not keep those after it from running on chip
         if (nres - k - n < kResMinSteps || o.ckpt_every < kResMinSteps) break;
@@ -463,7 +470,7 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
       void* tr = o.traces ? (char*)o.traces + (size_t)k * o.nrec * elem_size(dtype) : nullptr;
       double* en = o.energy ? o.energy + k : nullptr;
       cudaError_t e = cudaSuccess;
-      if (o.ckpt && due == 0) e = checkpoint(st, o, field_bytes, s);
+      if (now) e = checkpoint(st, o, field_bytes, s);
       int last = 0;
       if (e == cudaSuccess)
         e = res32 ? tsu::launch_step_res(sg, m->hx, m->hy, uu, vv, en, ews, n, s, o.nrec, o.rec_idx, tr, table, hold,

@@ -46,3 +46,14 @@ def test_short_stretch_before_a_checkpoint(dtype, nx, ny):
     # no stretch is long enough
     assert chip not in route(dtype, nx, ny, 40, nrec=9, every=7, first=3)
     same(dtype, nx, ny, 3, 40, 7, 9)
+
+
+@pytest.mark.parametrize("dtype,nx,ny", [("f32", 300, 200), ("f64", 129, 257)])
+def test_full_store(dtype, nx, ny):
+    """Behind the last slot no checkpoint cuts the call: 2 slots of 16 steps (states 1 and 17), then one launch."""
+    chip, one = ("k_leapfrog_res", "k_leapfrog") if dtype == "f32" else ("k_leapfrog_res64", "k_leapfrog64")
+    assert route(dtype, nx, ny, 100, nrec=9, every=16, slots=2) == {chip: 2}
+    assert route(dtype, nx, ny, 100, nrec=9, every=16, first=40, slots=2) == {chip: 1}
+    assert route(dtype, nx, ny, 103, nrec=9, every=16, first=13, slots=2) == {one: 3, chip: 1}
+    for first, steps in ((0, 100), (40, 100), (13, 103), (16, 50)):
+        same(dtype, nx, ny, first, steps, 16, 2)
