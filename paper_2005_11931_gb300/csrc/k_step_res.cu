@@ -814,6 +814,14 @@ bool res_fits(const StencilGeom& g, bool energy, bool rec, int32_t nrec, const E
   return res_plan(g, energy, rec, nrec, ews, &k, &rows);
 }
 
+// Tiles of 17 rows per warp take 16: with receivers 1900^2 (us per call on chip and in four-step passes) 74
+// and 65 at 8 steps, 95 and 92 at 12, 117 and 119 at 16; with a checkpoint every 8, 12 and 16 steps 81 and 69,
+// 98 and 94, 116 and 118 per interval.  At up to 14 rows 8 are enough (1800^2 54 and 61, 62 and 66).
+int64_t res_min_steps_recording(const StencilGeom& g, int64_t usual) {
+  int k = 0;
+  return res_rows(g.ny, g.ld, false, &k) > 0 && kResVariants[k].rows > kTmemRows ? 2 * usual : usual;
+}
+
 cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy, void* const u[2], void* const v[2],
                             double* energy, const EnergyWs& ews, int64_t nsteps, cudaStream_t s, int32_t nrec,
                             const int64_t* rec_idx, void* traces, bool table, bool hold, bool* ran, int* last) {

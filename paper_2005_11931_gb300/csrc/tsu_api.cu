@@ -316,7 +316,10 @@ static cudaError_t checkpoint(const tsu_state* st, const tsu_step_opts& o, size_
                          cudaMemcpyDeviceToDevice, s);
 }
 
-// calls of fewer steps are not worth reading the fields on chip and writing them back
+// Calls (or stretches between checkpoints) of fewer steps are not worth reading the fields on chip and writing
+// them back.  At 8 steps they are, us per call on chip and streaming: FP32 64^2 15 and 27, 769^2 18 and 30,
+// 1400^2 27 and 52, 2048^2 58 and 60, with the energy 20 and 39, 26 and 40, 39 and 72, 74 and 88; FP64 with the
+// energy 64^2 27 and 53, 740^2 157 and 203.
 static constexpr int64_t kResMinSteps = 8;
 
 int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, tsu_state* st, int64_t nsteps,
@@ -444,7 +447,9 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   const bool fits = o.kernel == 0 && o.rows == 0 && (res32 || res64) && (!o.traces || o.nrec <= tsu::kResMaxRec) &&
                     (res32 ? tsu::res_fits(sg, o.energy != nullptr, o.traces != nullptr, o.nrec, ews)
                            : tsu::res64_fits(sg, ews));
-  if (fits) {
+  const int64_t stretch = o.ckpt && o.ckpt_every < nsteps ? o.ckpt_every : nsteps;
+  const bool records = res32 && wtb_possible && (o.traces || o.ckpt);  // the four-step pass can as well
+  if (fits && stretch >= (records ? tsu::res_min_steps_recording(sg, kResMinSteps) : kResMinSteps)) {
     const int64_t nres = res32 && o.energy ? nsteps / 4 * 4 : nsteps;
     const bool hold = (o.reserved & 4) != 0;
     bool ran = true, table = true;
@@ -460,7 +465,7 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
       }
       if (n < kResMinSteps) {
         // a short stretch up to a checkpoint does not keep those after it from running on chip
-        if (nres - k - n < kResMinSteps || o.ckpt_every < kResMinSteps) break;
+        if (nres - k - n < kResMinSteps) break;
         TRY(one_step_passes(k + n));
         continue;
       }

@@ -72,6 +72,8 @@ cudaError_t launch_step_res(const StencilGeom& g, const void* hx, const void* hy
                             const int64_t* rec_idx, void* traces, bool table, bool hold, bool* ran, int* last);
 // whether such a call runs on chip on this device (rec: with traces)
 bool res_fits(const StencilGeom& g, bool energy, bool rec, int32_t nrec, const EnergyWs& ews);
+// the fewest steps worth a launch with receivers or checkpoints (usual: those of the other calls)
+int64_t res_min_steps_recording(const StencilGeom& g, int64_t usual);
 
 // The same for FP64 grids of up to about 750^2 in the standard form (k_step_res64.cu): u = u^n and
 // p = u^{n-1} are updated in place.

@@ -57,3 +57,16 @@ def test_full_store(dtype, nx, ny):
     assert route(dtype, nx, ny, 103, nrec=9, every=16, first=13, slots=2) == {one: 3, chip: 1}
     for first, steps in ((0, 100), (40, 100), (13, 103), (16, 50)):
         same(dtype, nx, ny, first, steps, 16, 2)
+
+
+def test_fewest_steps():
+    """With receivers or checkpoints the tiles of 17 rows per warp start at 16 steps, the others at 8; without
+    them all at 8."""
+    for n, fewest in ((1800, 8), (1900, 16), (2048, 16)):
+        assert route("f32", n, n, fewest, nrec=9) == {"k_leapfrog_res": 1}
+        assert route("f32", n, n, 48, every=fewest) == {"k_leapfrog_res": 48 // fewest}
+        assert route("f32", n, n, 8) == route("f32", n, n, 8, True) == {"k_leapfrog_res": 1}
+        assert "k_leapfrog_res" not in route("f32", n, n, fewest - 4, nrec=9)
+        assert "k_leapfrog_res" not in route("f32", n, n, 48, every=fewest - 4)
+    # an interval that the four-step pass cannot take
+    assert route("f32", 1900, 1900, 45, every=9) == {"k_leapfrog_res": 5}
