@@ -114,7 +114,7 @@ struct ResSmem {
   static constexpr bool kEs = ENERGY && !kLean && !kBatch;
   alignas(16) float er[kEr][ENERGY ? kResWarps * R : 1][32];
   float2 es[kEs ? kResK : 1][kEs ? kResThreads : 1];
-  float2 esw[kResK][kResWarps];
+  float3 esw[kResK][kResWarps];
   int2 rec[kResMaxRec];              // (row << 8 | column in the tile, receiver)
   // per warp: one row of u, or the values of its first and last output lanes on their way
   float4 stage[kLean ? 1 : kResWarps][kLean ? 1 : kStage];
@@ -207,12 +207,19 @@ __device__ __forceinline__ P4 tm_p4(const Tm8& d, int o) {
              pk(__uint_as_float(d.r[o + 2]), __uint_as_float(d.r[o + 3]))}};
 }
 
-// (s, lo) += (b, blo): the rounding error of the sum of the highs goes into the lows
-__device__ __forceinline__ void pair_add(float2& a, const float2 b) {
-  const float s = __fadd_rn(a.x, b.x), bb = __fsub_rn(s, a.x);
-  const float err = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
-  a.y = __fadd_rn(__fadd_rn(a.y, b.y), err);
-  a.x = s;
+// a += b, sums as three FP32 numbers: the errors of the highs go into the middles, theirs into the lows, about
+// 70 bits, where the other passes add in FP64 (two numbers, 46 bits, left energies off by up to 9e-15 from the
+// FP64 sums of the same chains, 64^2 to 2048^2; these by at most 6e-16, and cost 1 to 2 % more; FP64 itself
+// issues a warp instruction every 64 clocks)
+__device__ __forceinline__ float two_sum(float& s, const float b) {  // s += b; the error
+  const float t = __fadd_rn(s, b), z = __fsub_rn(t, s);
+  const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(b, z));
+  s = t;
+  return e;
+}
+__device__ __forceinline__ void sum_add(float3& a, const float3 b) {
+  const float e1 = two_sum(a.x, b.x), e2 = two_sum(a.y, b.y), e3 = two_sum(a.y, e1);
+  a.z = __fadd_rn(__fadd_rn(a.z, b.z), __fadd_rn(e2, e3));
 }
 
 template <int R, int RB, bool WIDE, bool ENERGY, bool REC>
@@ -599,14 +606,20 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
           if (t < ns) e[t] = LEAN ? a.es[((int64_t)cta * kResK + t) * kResThreads + tx] : sm.es[Smem::kEs ? t : 0][Smem::kEs ? tx : 0];
         }
       }
-      auto fold = [&](float2& keep, const float2& send, int o) {
-        pair_add(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, o), __shfl_xor_sync(0xffffffffu, send.y, o)));
+      auto fold = [&](float3& keep, const float3& send, int o) {
+        sum_add(keep, make_float3(__shfl_xor_sync(0xffffffffu, send.x, o), __shfl_xor_sync(0xffffffffu, send.y, o),
+                                  __shfl_xor_sync(0xffffffffu, send.z, o)));
+      };
+      // the first additions are of pairs: nothing in the lows to send
+      auto fold2 = [&](const float2& keep, const float2& send, int o) {
+        float3 k = make_float3(keep.x, keep.y, 0.f);
+        sum_add(k, make_float3(__shfl_xor_sync(0xffffffffu, send.x, o), __shfl_xor_sync(0xffffffffu, send.y, o), 0.f));
+        return k;
       };
       const bool h16 = lx & 16, h8 = lx & 8;
-      float2 k0 = h16 ? e[2] : e[0], k1 = h16 ? e[3] : e[1];
-      fold(k0, h16 ? e[0] : e[2], 16);
-      fold(k1, h16 ? e[1] : e[3], 16);
-      float2 k = h8 ? k1 : k0;
+      const float3 k0 = fold2(h16 ? e[2] : e[0], h16 ? e[0] : e[2], 16);
+      const float3 k1 = fold2(h16 ? e[3] : e[1], h16 ? e[1] : e[3], 16);
+      float3 k = h8 ? k1 : k0;
       fold(k, h8 ? k0 : k1, 8);
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1) fold(k, k, o);
@@ -614,12 +627,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_leapfrog_res(const ResArgs a
       if ((lx & 7) == 0) sm.esw[t][w] = k;
       __syncthreads();
       if (w == kResWarps - 1) {  // the CTA's sums
-        float2 x = sm.esw[t][lx & 7];
-        pair_add(x, sm.esw[t][(lx & 7) + 8]);
+        float3 x = sm.esw[t][lx & 7];
+        sum_add(x, sm.esw[t][(lx & 7) + 8]);
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) fold(x, x, o);
         if ((lx & 7) == 0 && t < ns)
-          a.part[((int64_t)p * kResK + t) * ncta + cta] = (double)x.x + (double)x.y;
+          a.part[((int64_t)p * kResK + t) * ncta + cta] = (double)x.x + ((double)x.y + (double)x.z);
       }
     } else {
       __syncthreads();
