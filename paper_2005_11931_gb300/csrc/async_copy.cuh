@@ -92,17 +92,12 @@ struct PollLimit {
   int* expired;
 };
 constexpr uint64_t kPollNs = 10000000000ull, kPollHookNs = 20000000ull;  // 10 s; test hook: 20 ms
-// Poll number `it` of a wait that began at t0: true when it has to be given up.  The check is a call of its
-// own: inlined, its registers spilled others of the steps (1800^2 with the energy 4.78 us per step instead
-// of 4.09).
-static __device__ __noinline__ bool poll_check(const PollLimit w, const uint64_t t0) {
+// whether a wait that began at t0 has to be given up (asked every 64 polls)
+__device__ __forceinline__ bool poll_over(const PollLimit& w, const uint64_t t0) {
   if (*(volatile int*)w.expired != 0) return true;
   if (global_ns() - t0 <= w.ns) return false;
   *(volatile int*)w.expired = 1;
   return true;
-}
-__device__ __forceinline__ bool poll_over(const PollLimit& w, const int it, const uint64_t t0) {
-  return (it & 63) == 63 && poll_check(w, t0);
 }
 constexpr int kPollCap = 1 << 30;  // iteration cap behind the wall-clock limit
 // bounded wait: true when the phase of this parity completed, false after limit_ns of wall-clock

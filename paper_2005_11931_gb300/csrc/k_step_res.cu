@@ -162,6 +162,9 @@ __device__ __forceinline__ bool item_try(const ResItem* d, float4& u, float4& v,
   for (int k = 0; k < 8; ++k) ok = ok && (uint32_t)(x[k] >> 32) == tag;
   return ok;
 }
+// a call of its own: inlined, its registers spilled others of the steps (1800^2 with the energy 4.78 us per
+// step instead of 4.09)
+__device__ __noinline__ bool item_over(const PollLimit w, const uint64_t t0) { return poll_over(w, t0); }
 // The item of pass `tag`, waited for with a bound (its CTA is resident: cooperative launch).  dead: a wait ran
 // out, now or before; what is not there is NaN, so that no result of it looks valid.
 __device__ __forceinline__ void item_get(const ResItem* d, float4& u, float4& v, const uint32_t tag, const PollLimit& w,
@@ -171,7 +174,7 @@ __device__ __forceinline__ void item_get(const ResItem* d, float4& u, float4& v,
     const uint64_t t0 = global_ns();
     for (int it = 0; it < kPollCap; ++it) {
       if (item_try(d, u, v, tag)) return;
-      if (poll_over(w, it, t0)) break;
+      if ((it & 63) == 63 && item_over(w, t0)) break;
     }
   }
   dead = true;

@@ -44,7 +44,7 @@ __device__ __forceinline__ double get64(ulonglong2 x, const ulonglong2* d, const
         dead = false;
         break;
       }
-      if (poll_over(w, it, t0)) break;
+      if ((it & 63) == 63 && poll_over(w, t0)) break;
     }
   }
   if (dead) return __longlong_as_double(0x7ff8000000000000ll);  // a wait ran out: nothing that follows is valid
