@@ -38,35 +38,57 @@ __device__ __forceinline__ double b64(const S64Geom& g, double fr, double fl, do
   return __fma_rn(g.cx, __dsub_rn(fr, fl), __dmul_rn(g.cy, __dsub_rn(gu, gd)));
 }
 
-// Sum of the CTAs' energy partials, by a CTA of kS64Warps warps; the result is thread 0's.  The additions near
-// the top of the tree make the rounding error of the whole sum (those of the many small sums below average
-// out), so here each one's error is kept and added at the end (Knuth's two-sum).  Relative error of energies
-// against binary128, rms over random fields at 101^2, 201^2, 400^2 and 1024^2: 0.8, 0.8, 0.7 and 0.6e-16
-// (on chip 0.8, 0.8, 0.8); with plain additions here 1.1, 1.1, 1.3 and 1.6e-16 (on chip 1.4, 1.4, 1.5);
-// plain here and every term compensated below (3 more FP64 operations per node) 1.0, 1.2, 1.1 and 1.4e-16.
+// Sum of the CTAs' energy partials (at most 2^30), by a CTA of kS64Warps warps; the result is thread 0's.  The
+// additions near the top of a tree make the rounding error of the whole sum (those of the many small sums
+// below average out), so this one is exact: every partial becomes an integer of 128 bits in units of 2^-92
+// times the largest's power of two, and the sum is rounded once.  Relative error of energies against
+// binary128, rms over random fields at 101^2, 201^2, 400^2 and 1024^2: 0.8, 0.8, 0.7 and 0.6e-16 (on chip 0.8,
+// 0.8, 0.8); with plain FP64 additions here 1.1, 1.1, 1.3 and 1.6e-16 (on chip 1.4, 1.4, 1.5); plain here and every term compensated
+// below (3 more FP64 operations per node) 1.0, 1.2, 1.1 and 1.4e-16.  Integers also because an FP64
+// instruction takes 64 clocks of a scheduler: keeping the errors in FP64 (two-sum) cost 2 us per sum.
 __device__ double partials_sum(const double* part, const int n) {
-  __shared__ double2 red[kS64Warps];
-  double s = 0.0, e = 0.0;
-  auto add = [&](const double x) {
-    const double t = __dadd_rn(s, x), z = __dsub_rn(t, s);
-    e = __dadd_rn(e, __dadd_rn(__dsub_rn(s, __dsub_rn(t, z)), __dsub_rn(x, z)));
-    s = t;
-  };
-  for (int q = threadIdx.x; q < n; q += kS64Warps * 32) add(__ldcg(part + q));
-  for (int k = 16; k > 0; k >>= 1) {
-    const double x = __shfl_down_sync(0xffffffffu, s, k), y = __shfl_down_sync(0xffffffffu, e, k);
-    add(x);
-    e = __dadd_rn(e, y);
-  }
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_double2(s, e);
+  __shared__ int top[kS64Warps];
+  __shared__ __int128 red[kS64Warps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  auto exponent = [](const double x) { return (int)(__double_as_longlong(x) >> 52) & 0x7ff; };
+  int e = 1;
+  for (int q = threadIdx.x; q < n; q += kS64Warps * 32) e = max(e, exponent(__ldcg(part + q)));
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0) top[w] = e;
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int q = 1; q < kS64Warps; ++q) {
-      add(red[q].x);
-      e = __dadd_rn(e, red[q].y);
-    }
-  const double t = __dadd_rn(s, e);
-  return isnan(t) ? s : t;  // an infinite sum has no error to add
+  for (int q = 0; q < kS64Warps; ++q) e = max(e, top[q]);
+  if (e == 0x7ff) {  // infinities or NaN
+    double s = 0.0;
+    if (threadIdx.x == 0)
+      for (int q = 0; q < n; ++q) s += __ldcg(part + q);
+    return s;
+  }
+  __int128 sum = 0;
+  for (int q = threadIdx.x; q < n; q += kS64Warps * 32) {
+    const double x = __ldcg(part + q);
+    const long long bits = __double_as_longlong(x);
+    const int f = exponent(x), down = e - max(f, 1);  // bits below the largest
+    const long long m = (bits & 0xfffffffffffffll) | (f > 0 ? 1ll << 52 : 0);
+    const __int128 v = down <= 40 ? (__int128)m << (40 - down) : (__int128)(down - 40 < 64 ? m >> (down - 40) : 0);
+    sum += bits < 0 ? -v : v;
+  }
+  for (int k = 16; k > 0; k >>= 1) {
+    const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)sum, k);
+    const long long hi = __shfl_down_sync(0xffffffffu, (long long)(sum >> 64), k);
+    sum += ((__int128)hi << 64) | lo;
+  }
+  if (lane == 0) red[w] = sum;
+  __syncthreads();
+  if (threadIdx.x != 0) return 0.0;
+  for (int q = 1; q < kS64Warps; ++q) sum += red[q];
+  // the top 64 bits (those below them only decide ties), rounded once
+  unsigned __int128 mag = sum < 0 ? (unsigned __int128)-sum : (unsigned __int128)sum;
+  const unsigned long long hi = (unsigned long long)(mag >> 64);
+  const int drop = hi ? 64 - __clzll((long long)hi) : 0;
+  unsigned long long m = (unsigned long long)(mag >> drop);
+  if (drop && (mag & (((unsigned __int128)1 << drop) - 1))) m |= 1;
+  const double s = ldexp(__ull2double_rn(m), drop + e - 1023 - 52 - 40);
+  return sum < 0 ? -s : s;
 }
 
 // FORM 0: standard (p = u^{n-1}, out = u^{n+1}, may be written over p); FORM 1: increment (p = v^n updated
