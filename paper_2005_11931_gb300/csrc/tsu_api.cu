@@ -445,8 +445,9 @@ int tsu_step_n(const tsu_grid* g, int dtype, double tau, const tsu_medium* m, ts
   const bool res32 = flow_base && !(o.energy && o.ckpt);
   const bool res64 = dtype == TSU_F64 && st->form == TSU_FORM_STANDARD && have_ws;
   const bool fits = o.kernel == 0 && o.rows == 0 && (res32 || res64) && (!o.traces || o.nrec <= tsu::kResMaxRec) &&
-                    (res32 ? tsu::res_fits(sg, o.energy != nullptr, o.traces != nullptr, o.nrec, ews)
-                           : tsu::res64_fits(sg, ews));
+                    (!o.ckpt ? true  // the launch itself says so
+                     : res32 ? tsu::res_fits(sg, o.energy != nullptr, o.traces != nullptr, o.nrec, ews)
+                             : tsu::res64_fits(sg, ews));
   const int64_t stretch = o.ckpt && o.ckpt_every < nsteps ? o.ckpt_every : nsteps;
   const bool records = res32 && wtb_possible && (o.traces || o.ckpt);  // the four-step pass can as well
   if (fits && stretch >= (records ? tsu::res_min_steps_recording(sg, kResMinSteps) : kResMinSteps)) {
