@@ -153,8 +153,11 @@ typedef struct {
                        through tsu_sync_status); auto (with rows = 0) keeps grids that fit on chip there for
                        the whole call, or up to the next checkpoint, in one cooperative launch (FP32
                        in the increment form with nbuf = 4 up to about 2000^2, FP64 in the standard
-                       form up to about 750^2; a workspace, at most 512 receivers, at least 8 steps;
-                       its waits are bounded as kernel 4's); else kernel 4 where it can run and its
+                       form up to about 750^2; a workspace, at most 512 receivers, at least 8 steps
+                       in the call and between checkpoints; in FP32 not with the energy and
+                       checkpoints together, with the energy and receivers up to about 1750^2, and
+                       from about 1890^2 on with receivers or checkpoints at least 16 steps;
+                       its waits are bounded as kernel 4's, by 10 s); else kernel 4 where it can run and its
                        tiles number between half and 6 times the device's resident warps (FP32 grids
                        of about 2K to 12K per side), else kernel 2 (tdepth 4) whenever it can.  All
                        kernels round every operation the same way, so the states do not depend on

@@ -13,7 +13,7 @@
 //    (step64_rows);
 //  - the fields of four rows are loaded before the first of them is used.
 // Measured (GB300, us per step, before and after): with the energy 201^2 13.9 and 6.2 (the launch: a step
-// takes a multiple of 2.05 us back to back), 2048^2 196 and 139 (0.83 of the FP64 pipe's rate);
+// takes a multiple of 2.05 us back to back), 2048^2 196 and 127 (the FP64 pipe 84 % active);
 // without it 2048^2 114 and 97; a 257^2 gradient of 300 steps 9.5 and 5.2 ms.  Programmatic dependent
 // launches were slower (201^2 11.1): the early CTAs doubled up on some SMs.
 #include "stencil_common.cuh"

@@ -12,12 +12,13 @@
 // and the pass that wrote it, so the reader polls the data themselves (a flag behind a fence took
 // 1.30 us per step at 64^2 with the energy instead of 1.05).
 //
-// What bounds it: the FP32 pipe and instruction issue (about 90 warp instructions per row of 128
-// nodes and step, 46 of them FP32 arithmetic; streaming tiles through shared memory and register
-// windows, as k_step_wtb.cu does, takes 100 to 176), and one exchange, about 2 us, per four steps.
+// What bounds it: the FP32 pipe and instruction issue (without the energy 59 warp instructions per row of
+// 128 nodes and step at 8 rows per warp, 61 at 17, 33 of them FP32 arithmetic; streaming tiles through
+// shared memory and register windows, as k_step_wtb.cu does, takes 100 to 176), and one exchange, about
+// 2 us, per four steps.
 // Measured (GB300, us per step, before and after): 769^2 with receivers 4.1 and 1.35; 1024^2 3.6 and
 // 1.43, 1400^2 4.6 and 1.9, 2048^2 5.9 and 4.7; with the energy 1003 x 517 4.8 and 1.7, 1024^2 4.9 and
-// 1.8, 1536^2 5.7 and 3.0, 2048^2 6.85 and 6.05.
+// 1.8, 1536^2 5.7 and 3.1, 2048^2 6.85 and 6.1.
 //
 // All warps run the row code in step (a barrier per step): when only neighbouring warps waited for
 // each other they drifted apart, and the unrolled code of all of them no longer fitted the
@@ -730,7 +731,10 @@ constexpr ResVariant res_variant() {
   if constexpr (!res_lean(R, ENERGY)) v.kern[1] = k_leapfrog_res<R, RB, WIDE, ENERGY, true>;
   return v;
 }
-// without the energy, then with it
+// Without the energy, then with it.  A grid takes the fewest rows per warp that hold it; between 8 and 17 not
+// every count is built, so some grids carry rows they do not need (1900^2 17: 4.62 us per step without the
+// energy, where 1800^2 takes 3.08 at 14).  17 is one row more than tensor memory holds; it is what 2048 rows
+// in 8 chunks need.
 const ResVariant kResVariants[] = {
     res_variant<2, 2, false, false>(),  res_variant<3, 3, false, false>(), res_variant<4, 2, false, false>(),
     res_variant<5, 2, true, false>(),  res_variant<6, 2, true, false>(), res_variant<7, 2, true, false>(),

@@ -57,7 +57,7 @@ inline size_t flow_bytes(int64_t tiles) {
 
 // The resident pass (k_step_res.cu): one CTA per SM, every step of a call in one cooperative launch,
 // for grids whose fields fit on chip.  Its region of the workspace holds the rims that the CTAs
-// exchange and a ring of energy partials.
+// exchange and the energy partials of a launch.
 constexpr int kResMaxCtas = 160;
 constexpr int32_t kResMaxRec = 512;  // receivers a CTA keeps in its list
 size_t res_bytes(int64_t ny, int64_t ld);  // 0: the grid does not fit
