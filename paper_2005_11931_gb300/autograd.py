@@ -63,7 +63,7 @@ class TsunamiFn(torch.autograd.Function):
         tsu.tsu_observe(g, code, cfg.tau, med, st, None, cfg.rec_idx, traces[S - 1], ws, ws_b)
         ctx.save_for_backward(hx, hy, u0, ckpt)
         ctx.cfg = cfg
-        ctx.status_ws = ws  # holds the status word of the run's bounded waits: sync_status
+        ctx.status = ws[:256].clone()  # with the status word of the run's bounded waits (sync_status); ws is freed here
         return traces
 
     @staticmethod
@@ -101,6 +101,6 @@ def sync_status(traces: torch.Tensor, stream=None):
     recorded ``traces`` (as returned by tsunami_traces, with a gradient) ran out.  Nothing synchronises
     otherwise: such a run leaves NaN in the fields, and in the traces and gradients that depend on them."""
     fn = traces.grad_fn
-    if not hasattr(fn, "status_ws"):
+    if not hasattr(fn, "status"):
         raise ValueError("traces must be the tensor tsunami_traces returned for inputs that require a gradient")
-    tsu.tsu_sync_status(fn.status_ws, fn.status_ws.numel(), stream)
+    tsu.tsu_sync_status(fn.status, fn.status.numel(), stream)
